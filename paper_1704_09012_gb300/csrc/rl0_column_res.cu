@@ -35,7 +35,7 @@
 
 #include "rl0_common.cuh"
 #include "rl0_device.cuh"
-#include "rl0_mma.cuh"
+#include "rl0_resolve.cuh"
 #include "rl0_round.cuh"
 
 #define RL0_RES_CHUNK 32768u            // bytes per bulk copy
@@ -43,15 +43,6 @@
 #define RL0_RES_MAX_NT 1024
 
 namespace {
-
-struct ResShared {
-    Series pe;
-    unsigned long long bar;             // completion of the bulk copies
-    int count, last;
-    unsigned total, ubase, fbase;
-    int dn;                             // this CTA's change of the nonzero count
-    unsigned nnz0;                      // |supp x_hat| at the round's start
-};
 
 // A survivor staged in shared memory: its column, candidate slots, x_j, the
 // (r, p_z) of its rows (x_j and (r, p_z) copied with cp.async) and its row ids
@@ -102,56 +93,6 @@ __device__ __forceinline__ bool mbar_try_wait_bounded(unsigned bar, unsigned par
     return false;
 }
 
-// Resolve scratch, laid over the code region once the stream is done: a
-// batch of NT listed columns and their candidate items (at most DMAX each).
-template <int DMAX, int NT, bool LEARNED = false>
-struct ResScratch {
-    float r[DMAX][NT];                   // FP32 residuals of the batch's columns
-    float nz[NT], rhs[NT];
-    unsigned off[NT];                    // first item of each column
-    unsigned short it_e[NT * DMAX];      // item -> column in the batch
-    unsigned char it_s[NT * DMAX];       // item -> slot (descending within a column)
-    unsigned char it_ok[NT * DMAX];
-    float it_w[NT * DMAX];
-    float it_sc[NT * DMAX];              // n_e - n_z of the item
-    float feat[LEARNED ? NT : 1][RL0_NFEAT];   // learned scorer: features of the items that pass the
-    unsigned short fidx[LEARNED ? NT : 1];     // exact tests (compact, NT items at a time) and their items
-    float q[NT][DMAX];                   // q_e of (item, slot l), NT items at a time
-    unsigned wsum[NT / 32];
-    int nf;
-};
-
-// Exclusive prefix over the CTA of v (NT threads, all of them call it);
-// *total (shared) gets the sum.  wsum: NT / 32 shared words.
-template <int NT>
-__device__ __forceinline__ unsigned cta_exclusive_scan(unsigned v, unsigned *wsum, unsigned *total)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const unsigned w = (lane < NT / 32) ? wsum[lane] : 0u;
-        unsigned wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned t = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += t;
-        }
-        if (lane < NT / 32) wsum[lane] = wi - w;
-        if (lane == 31) *total = wi;
-    }
-    __syncthreads();
-    const unsigned r = wsum[warp] + incl - v;
-    __syncthreads();
-    return r;
-}
-
 // One round's column score up to the CTA's commit (load, stream, resolve).
 // DMAX slots per column; EXACT: d == DMAX (the slot guards fold away).
 // cur, round: the decode state's accepted buffer and round (read by the caller).
@@ -166,7 +107,7 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     const int d = EXACT ? DMAX : a.d;
     const unsigned short *s_code = (const unsigned short *)dsm;
     const float *s_pz = (const float *)(dsm + a.res_pz_off);
-    ResShared &S = *(ResShared *)(dsm + a.res_s_off);
+    ColState &S = *(ColState *)(dsm + a.res_s_off);
     // this CTA's columns: [lo, hi), equal shares of n
     const int lo = (int)(((long long)blockIdx.x * n) / gridDim.x);
     const int hi = (int)(((long long)(blockIdx.x + 1) * n) / gridDim.x);
@@ -392,15 +333,14 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     if (LEARNED && tid == 0) R.nf = 0;              // first read after the batch's barriers
     const float alpha = ctx->alpha;
     for (int b0 = 0; b0 < count; b0 += NT) {
-        // one thread per listed column: FP32 residuals, exact candidates
+        // one thread per listed column: its FP32 residuals
         const int e = b0 + tid;
         const bool act = e < count;
         int j = 0;
-        unsigned cand = 0u;
+        unsigned cm = 0u;
         float old = 0.0f;
+        float2 v[DMAX];
         if (act) {
-            float2 v[DMAX];
-            unsigned cm;
             if (e < qcap) {
                 const ResEntry<DMAX> &q = sq[e];
                 j = q.j;
@@ -416,170 +356,18 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
 #pragma unroll
                 for (int s = 0; s < DMAX; ++s) v[s] = (s < d) ? __ldg(rz + __ldcg(ent + 2 + s)) : make_float2(0.0f, 0.0f);
             }
-            float nz = 0.0f, rhs = 0.0f;
-#pragma unroll
-            for (int s = 0; s < DMAX; ++s) {
-                if (s < d) {
-                    nz += IND ? (fabsf(v[s].x) <= th.tz ? 1.0f : 0.0f) : v[s].y;
-                    rhs += fabsf(v[s].x);
-                    // the code bound's candidates that are anchors: a superset of
-                    // the passing anchors, each then tested exactly below
-                    if (((cm >> s) & 1u) && fabsf(v[s].x) >= th.ta) cand |= 1u << s;
-                }
-                R.r[s][tid] = (s < d) ? v[s].x : 0.0f;
-            }
-            R.nz[tid] = nz;
-            R.rhs[tid] = rhs;
         }
-        // one item per candidate (column, slot), a column's slots in descending order
-        const unsigned nc = (unsigned)__popc(cand);
-        const unsigned off = cta_exclusive_scan<NT>(nc, R.wsum, &S.total);
-        const unsigned nitems = S.total;
-        {
-            unsigned c = cand, q = off;
-            while (c) {
-                const int sl = 31 - __clz(c);
-                c &= ~(1u << sl);
-                R.it_e[q] = (unsigned short)tid;
-                R.it_s[q] = (unsigned char)sl;
-                ++q;
-            }
-        }
-        __syncthreads();
-        // eval_anchor's arithmetic in two steps, so that an item's d posteriors
-        // are evaluated side by side (one per thread) rather than one after
-        // another: q_e of every (item, l), then each item's sums in slot order
-        for (unsigned k0 = 0; k0 < nitems; k0 += NT) {
-            const unsigned kn = min(nitems - k0, (unsigned)NT);
-            for (unsigned p = tid; p < kn * (unsigned)d; p += NT) {
-                const unsigned kk = p / (unsigned)d, l = p % (unsigned)d;
-                const int ee = R.it_e[k0 + kk], sl = R.it_s[k0 + kk];
-                const float rs = R.r[sl][ee], rl = R.r[l][ee];
-                R.q[kk][l] = IND ? (fabsf(rs - rl) <= th.te ? 1.0f : 0.0f) : series_eval(S.pe, rs - rl);
-            }
-            __syncthreads();
-            for (unsigned kk = tid; kk < kn; kk += NT) {
-                const unsigned k = k0 + kk;
-                const int ee = R.it_e[k];
-                float ne = 0.0f, num = 0.0f;
-                for (int l = 0; l < d; ++l) {
-                    const float rl = R.r[l][ee];
-                    const float q = R.q[kk][l];
-                    ne += q;
-                    num += rl * q;
-                }
-                const float w = num / ne;
-                float lhs = 0.0f;
-                for (int l = 0; l < d; ++l) lhs += fabsf(R.r[l][ee] - w);
-                if constexpr (LEARNED) {
-                    // the learned scorer: the l1 test and n_e - n_z >= 1.5 here; the
-                    // features of the items that pass go to a compact list, whose
-                    // logits the network takes below
-                    const bool ok = lhs <= R.rhs[ee] && ne - R.nz[ee] >= ctx->learned_need;
-                    R.it_ok[k] = ok ? 1 : 0;
-                    if (ok) {
-                        AnchorEval E;
-                        E.ne = ne;
-                        E.w = w;
-                        E.lhs = lhs;
-                        float f[RL0_NFEAT];
-                        candidate_features(&R.r[0][ee], NT, d, E, R.nz[ee], R.rhs[ee], ctx->inv_sn, th.t, ctx->drho,
-                                           f);
-                        const int p = atomicAdd(&R.nf, 1);
-#pragma unroll
-                        for (int q = 0; q < RL0_NFEAT; ++q) R.feat[p][q] = f[q];
-                        R.fidx[p] = (unsigned short)kk;
-                    }
-                } else {
-                    R.it_ok[k] = (lhs <= R.rhs[ee] && ne - R.nz[ee] >= alpha) ? 1 : 0;
-                }
-                R.it_w[k] = w;
-                R.it_sc[k] = ne - R.nz[ee];
-            }
-            __syncthreads();
-            if constexpr (LEARNED) {
-                // the passing items' logits, 16 per warp on the tensor cores
-                const unsigned nf = (unsigned)R.nf;
-                const __nv_bfloat16 *wb = (const __nv_bfloat16 *)ctx->mlp;
-                for (unsigned t0 = (unsigned)(tid >> 5) * 16u; t0 < nf; t0 += (NT / 32) * 16u) {
-                    auto f = [&](int r, int i) { return (t0 + r < nf) ? R.feat[t0 + r][i] : 0.0f; };
-                    float lo, hi;
-                    warp_mlp_logits16(f, wb, &lo, &hi);
-                    if ((tid & 3) == 0) {
-                        const unsigned gr = (unsigned)((tid & 31) >> 2);
-                        if (t0 + gr < nf && !(lo >= ctx->logit_thr)) R.it_ok[k0 + R.fidx[t0 + gr]] = 0;
-                        if (t0 + gr + 8 < nf && !(hi >= ctx->logit_thr)) R.it_ok[k0 + R.fidx[t0 + gr + 8]] = 0;
-                    }
-                }
-                __syncthreads();
-                if (tid == 0) R.nf = 0;                // read again only after the next batch's barriers
-            }
-        }
-        // each column: its first passing item is its highest passing slot (the
-        // last passing anchor in row order); with anchor_rule 1 the passing item
-        // of largest n_e - n_z, ties to the lower slot (items come highest first)
-        int best = -1;
-        float bw = 0.0f, bsc = 0.0f;
-        for (unsigned q = 0; q < nc; ++q)
-            if (R.it_ok[off + q]) {
-                if (rule == 0) {
-                    best = R.it_s[off + q];
-                    bw = R.it_w[off + q];
-                    break;
-                }
-                if (best < 0 || R.it_sc[off + q] >= bsc) {
-                    best = R.it_s[off + q];
-                    bw = R.it_w[off + q];
-                    bsc = R.it_sc[off + q];
-                }
-            }
-        const bool pass = best >= 0;
-        float nv = old;
-        if (pass) {
-            nv = old + bw;
-            ctx->x[j] = nv;
-        }
-        if (passed && act) passed[j] = pass ? 1 : 0;
-        // a column that became nonzero takes its rows' fresh-bucket slots now,
-        // so that those atomics travel with the commit's below
-        const bool fresh = pass && old == 0.0f && nv != 0.0f;
-        int rid[DMAX], slot[DMAX];
-        if (fresh) {
+        auto rows = [&](int *rid) {
             if (e < qcap) {
 #pragma unroll
-                for (int s2 = 0; s2 < DMAX; ++s2) rid[s2] = (s2 < d) ? sq[e].rid[s2] : 0;
+                for (int s = 0; s < DMAX; ++s) rid[s] = (s < d) ? sq[e].rid[s] : 0;
             } else {
                 const int *ent = seg + (size_t)e * (DMAX + 2);
 #pragma unroll
-                for (int s2 = 0; s2 < DMAX; ++s2) rid[s2] = (s2 < d) ? __ldcg(ent + 2 + s2) : 0;
+                for (int s = 0; s < DMAX; ++s) rid[s] = (s < d) ? __ldcg(ent + 2 + s) : 0;
             }
-            bucket_slots<DMAX>(a, rid, d, slot);
-        }
-        // the batch's commit: one global atomic per counter
-        const unsigned pf = cta_exclusive_scan<NT>((pass ? 0x10000u : 0u) | (fresh ? 1u : 0u), R.wsum, &S.total);
-        const unsigned tpf = S.total;
-        // entries that became zero; the fresh ones are the scan's low field
-        const int ngone = __syncthreads_count(pass && old != 0.0f && nv == 0.0f);
-        if (tid == 0) {
-            const int nup = (int)(tpf & 0xffffu);
-            S.dn += nup - ngone;                   // added to the ticket at the end
-            if (ngone) atomicAdd(&st->zeroed, (unsigned)ngone);
-            const unsigned long long old2 = (tpf != 0u) ? take_upd_list(st, tpf >> 16, tpf & 0xffffu) : 0ull;
-            S.ubase = (unsigned)(old2 >> 32);
-            S.fbase = (unsigned)old2;
-        }
-        __syncthreads();
-        if (pass) {
-            UndoEntry u;
-            u.j = j;
-            u.old = old;
-            a.ulog[S.ubase + (pf >> 16)] = u;
-        }
-        if (fresh) {
-            a.list[S.fbase + (pf & 0xffffu)] = j;
-            bucket_store<DMAX>(a, j, rid, d, slot);
-        }
-        __syncthreads();                           // the scratch is reused by the next batch
+        };
+        resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, d, rule, alpha, passed, R, S, act, j, cm, old, v, rows);
     }
     return true;
 }
@@ -590,7 +378,7 @@ __global__ void __launch_bounds__(NT, 1) k_column_score_res(KArgs a)
     extern __shared__ __align__(16) unsigned char dsm[];
     if (!column_phase<DMAX, IND, EXACT, NT, LEARNED>(a, dsm)) return;     // the decode is done
     // the codes are no longer needed: their bytes become H_k's scratch
-    ResShared &S = *(ResShared *)(dsm + a.res_s_off);
+    ColState &S = *(ColState *)(dsm + a.res_s_off);
     HkShared &hk = *(HkShared *)dsm;
     unsigned *suf = (unsigned *)(dsm + ((sizeof(HkShared) + 15) & ~(size_t)15));
     last_cta_hk_tick<NT>(a, a.ctx, hk, suf, &S.last, S.dn, S.nnz0);
@@ -603,11 +391,12 @@ template <int DMAX, bool EXACT> struct ResNT {
     static constexpr int value = DMAX <= 16 ? 512 : 256;
 };
 
+// (the limit set is the device's, not this expander's size: the attribute
+// belongs to the kernel, which expanders of other sizes launch too)
 template <int DMAX, bool EXACT>
-bool res_attr(unsigned smem)
+bool res_attr(int sm)
 {
     constexpr int NT = ResNT<DMAX, EXACT>::value;
-    const int sm = (int)smem;
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if (cudaFuncSetAttribute(k_column_score_res<DMAX, false, EXACT, NT, false>, at, sm) != cudaSuccess ||
         cudaFuncSetAttribute(k_column_score_res<DMAX, true, EXACT, NT, false>, at, sm) != cudaSuccess ||
@@ -657,7 +446,7 @@ void rl0_res_setup(const rl0_expander *A, KArgs *a)
     const unsigned region = res_region_bytes(A->m, nt, res_scratch_bytes(A->d));
     a->res_pz_off = region;
     a->res_s_off = region + 4u * RL0_PZ_BINS;
-    a->res_q_off = (a->res_s_off + (unsigned)sizeof(ResShared) + 15u) & ~15u;
+    a->res_q_off = (a->res_s_off + (unsigned)sizeof(ColState) + 15u) & ~15u;
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, A->device) != cudaSuccess) {
         cudaGetLastError();
@@ -671,11 +460,11 @@ void rl0_res_setup(const rl0_expander *A, KArgs *a)
     a->res_smem = a->res_q_off + (unsigned)a->res_qcap * eb;
     bool ok = false;
     switch (res_variant(A->d)) {
-    case 6: ok = res_attr<6, true>(a->res_smem); break;
-    case 7: ok = res_attr<7, true>(a->res_smem); break;
-    case 8: ok = (A->d == 8) ? res_attr<8, true>(a->res_smem) : res_attr<8, false>(a->res_smem); break;
-    case 16: ok = res_attr<16, false>(a->res_smem); break;
-    default: ok = res_attr<32, false>(a->res_smem); break;
+    case 6: ok = res_attr<6, true>(optin); break;
+    case 7: ok = res_attr<7, true>(optin); break;
+    case 8: ok = (A->d == 8) ? res_attr<8, true>(optin) : res_attr<8, false>(optin); break;
+    case 16: ok = res_attr<16, false>(optin); break;
+    default: ok = res_attr<32, false>(optin); break;
     }
     if (!ok) return;
     const long long ntiles = rl0_div_up(A->n, nt);

@@ -174,6 +174,7 @@ struct rl0_expander {
     int last_log_rounds;      // rounds recorded by the last rl0_decode
     void *events;             // CUDA events used to time decodes
     void *table_cache;        // host tables of the last parameter set
+    void *kargs;              // the round kernels' argument block (KArgs)
     int wait_test;            // rl0_expander_set_wait_polls: override the first bounded wait
     unsigned wait_polls;
 };

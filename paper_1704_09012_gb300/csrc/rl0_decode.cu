@@ -170,198 +170,6 @@ __global__ void k_list_count_from_support(KArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// Column score: Algorithm 2's loop over j in [n] and i in N(j).
-//
-// One thread per column.  Fast path (registers only): the anchors
-// (|r_i| >= ta) and, for every anchor, the mask of rows within reach of it --
-// |r_i - r_l| <= te for the 0/1 scores, or <= the 2^-40 cut of p_e for the
-// continuous scores, where n_e <= 1 + popc(mask).  An anchor whose bound
-// cannot reach n_e - n_z >= alpha is dropped here; for the 0/1 scores the
-// bound is n_e itself.  Slow path (rare): the surviving anchors get the exact
-// n_e, omega and l1 test from residuals kept in shared memory, scored by the
-// whole CTA from each column's highest slot down until one passes (that one is
-// the last passing anchor in row order, whose omega the column takes).
-// ---------------------------------------------------------------------------
-template <int DMAX> struct ColBlock { static constexpr int value = DMAX <= 8 ? 256 : (DMAX <= 16 ? 128 : 64); };
-
-// Shared memory of the column kernels.  H_k's scratch (used by the launch's
-// last CTA after its tiles) shares the bytes of the candidate queue.
-template <int DMAX, int NT, bool LEARNED>
-struct ColShared {
-    union {
-        struct {
-            float r[DMAX][NT];                 // residuals of columns with candidates
-            float nz[NT], rhs[NT];
-            unsigned short q[NT];              // this pass's queue: (column lane << 5) | slot
-            float score[NT], w[NT];
-            unsigned char ok[NT];
-            float f[LEARNED ? RL0_NFEAT : 1][LEARNED ? NT : 1];   // features of the candidates that pass
-            unsigned short fq[LEARNED ? NT : 1];                  // their queue positions
-        } c;
-        struct {
-            HkShared hk;
-            unsigned suf[NT];
-        } h;
-    };
-    Series pe;
-    int nq, nf;
-    int last;
-};
-
-template <int DMAX, bool IND, bool LEARNED, int NT>
-__device__ __forceinline__ void col_setup(const DecodeCtx *ctx, ColShared<DMAX, NT, LEARNED> &S)
-{
-    const int tid = threadIdx.x;
-    if (tid == 0) {
-        S.nq = 0;
-        S.nf = 0;
-        if (!IND) S.pe = ctx->pe;
-    }
-    // (these shared copies are first read after a barrier of the tile body)
-}
-
-// One tile of NT columns starting at j0.  gather(row) returns (r_row, p_z(r_row)).
-template <int DMAX, bool IND, bool LEARNED, int NT, class Gather>
-__device__ __forceinline__ void score_tile(const KArgs &a, const DecodeCtx *ctx, const RoundThr &th, int j0,
-                                           Gather gather, ColShared<DMAX, NT, LEARNED> &S)
-{
-    const int tid = threadIdx.x;
-    const int n = a.n, d = a.d;
-    const int j = j0 + tid;
-    const bool active = j < n;
-    const float alpha = ctx->alpha;
-
-    float r[DMAX];
-    float nz = 0.0f, rhs = 0.0f;
-#pragma unroll
-    for (int s = 0; s < DMAX; ++s) {
-        r[s] = 0.0f;
-        if (s < d && active) {
-            const float2 v = gather(__ldg(a.rows_sm + (size_t)s * n + j));
-            r[s] = v.x;
-            nz += IND ? (fabsf(v.x) <= th.tz ? 1.0f : 0.0f) : v.y;
-            rhs += fabsf(v.x);
-        }
-    }
-    const float need = LEARNED ? (IND ? ctx->learned_need : ctx->learned_need - 1e-3f) : (IND ? alpha : alpha - 1e-3f);
-    unsigned cand = active ? anchor_candidates<DMAX, IND>(r, d, th.ta, IND ? th.te : ctx->pe.cut, ctx->pe_b1,
-                                                          ctx->pe_c1, nz, need) : 0u;
-    if (cand) {
-#pragma unroll
-        for (int s = 0; s < DMAX; ++s) S.c.r[s][tid] = r[s];
-        S.c.nz[tid] = nz;
-        S.c.rhs[tid] = rhs;
-    }
-    int best = -1;
-    float bw = 0.0f, bsc = 0.0f;
-    while (__syncthreads_or(cand != 0u)) {
-        int my = -1, ms = 0;
-        if (cand) {
-            ms = 31 - __clz(cand);                  // highest remaining slot first
-            cand &= ~(1u << ms);
-            my = atomicAdd(&S.nq, 1);
-            S.c.q[my] = (unsigned short)((tid << 5) | ms);
-        }
-        __syncthreads();
-        const int nq = S.nq;
-        if (LEARNED) {
-            // the learned scorer's logit replaces n_e - n_z >= alpha: each queued
-            // candidate's exact l1 test and n_e - n_z >= 1.5 first; the features
-            // of those that pass go to a compact list, whose logits the MLP takes
-            // 16 per warp on the tensor cores (rl0_mma.cuh: the arithmetic of
-            // rl0_mlp_forward); a candidate passes when its logit reaches the
-            // threshold
-            for (int e = tid; e < nq; e += NT) {
-                const int owner = S.c.q[e] >> 5, s = S.c.q[e] & 31;
-                const AnchorEval E = eval_anchor<IND>(&S.c.r[0][owner], NT, d, s, th.te, S.pe);
-                S.c.ok[e] = 0;
-                S.c.score[e] = 0.0f;
-                S.c.w[e] = E.w;
-                if (E.lhs <= S.c.rhs[owner] && E.ne - S.c.nz[owner] >= ctx->learned_need) {
-                    const int p = atomicAdd(&S.nf, 1);
-                    float f[RL0_NFEAT];
-                    candidate_features(&S.c.r[0][owner], NT, d, E, S.c.nz[owner], S.c.rhs[owner], ctx->inv_sn,
-                                       th.t, ctx->drho, f);
-#pragma unroll
-                    for (int q = 0; q < RL0_NFEAT; ++q) S.c.f[q][p] = f[q];
-                    S.c.fq[p] = (unsigned short)e;
-                }
-            }
-            __syncthreads();
-            const int nf = S.nf;
-            const __nv_bfloat16 *wb = (const __nv_bfloat16 *)ctx->mlp;
-            for (int e0 = (tid >> 5) * 16; e0 < nf; e0 += (NT / 32) * 16) {
-                auto f = [&](int r, int i) { return (e0 + r < nf) ? S.c.f[i][e0 + r] : 0.0f; };
-                float lo, hi;
-                warp_mlp_logits16(f, wb, &lo, &hi);
-                if ((tid & 3) == 0) {
-                    const int gr = (tid & 31) >> 2;
-                    if (e0 + gr < nf) {
-                        const int e = S.c.fq[e0 + gr];
-                        S.c.score[e] = lo;
-                        S.c.ok[e] = (lo >= ctx->logit_thr) ? 1 : 0;
-                    }
-                    if (e0 + gr + 8 < nf) {
-                        const int e = S.c.fq[e0 + gr + 8];
-                        S.c.score[e] = hi;
-                        S.c.ok[e] = (hi >= ctx->logit_thr) ? 1 : 0;
-                    }
-                }
-            }
-        } else {
-            for (int e = tid; e < nq; e += NT) {
-                const int owner = S.c.q[e] >> 5, s = S.c.q[e] & 31;
-                float sc, w;
-                S.c.ok[e] = score_anchor<IND>(&S.c.r[0][owner], NT, d, s, th.te, S.pe, S.c.nz[owner], S.c.rhs[owner],
-                                              alpha, &sc, &w) ? 1 : 0;
-                S.c.score[e] = sc;
-                S.c.w[e] = w;
-            }
-        }
-        __syncthreads();
-        if (my >= 0 && S.c.ok[my]) {
-            if (ctx->anchor_rule == 0) {            // the first pass from the top is the last passing
-                best = ms;                          // anchor in row order: it stands, the rest is moot
-                bw = S.c.w[my];
-                cand = 0u;
-            } else if (best < 0 || S.c.score[my] >= bsc) {   // largest n_e - n_z; slots come highest
-                best = ms;                                   // first, so >= leaves ties to the lower row
-                bw = S.c.w[my];
-                bsc = S.c.score[my];
-            }
-        }
-        if (tid == 0) {
-            S.nq = 0;
-            S.nf = 0;
-        }
-    }
-    commit_column(a, ctx, j, active, best, bw);
-}
-
-template <int DMAX, int NT, bool LEARNED>
-__device__ __forceinline__ void col_last_cta(const KArgs &a, const DecodeCtx *ctx, ColShared<DMAX, NT, LEARNED> &S)
-{
-    last_cta_hk<NT>(a, ctx, S.h.hk, S.h.suf, &S.last);
-}
-
-template <int DMAX, bool IND, bool LEARNED>
-__global__ void __launch_bounds__(ColBlock<DMAX>::value) k_column_score(KArgs a)
-{
-    constexpr int NT = ColBlock<DMAX>::value;
-    __shared__ ColShared<DMAX, NT, LEARNED> S;
-    const DecodeState *st = a.st;
-    pdl_wait();                                    // the previous rebuild's r, x and state
-    pdl_launch_dependents();
-    if (st->done) return;
-    const DecodeCtx *ctx = a.ctx;
-    const float2 *__restrict__ rz = st->cur ? a.rz1 : a.rz0;
-    const RoundThr th = a.thr[st->round];
-    col_setup<DMAX, IND, LEARNED, NT>(ctx, S);
-    score_tile<DMAX, IND, LEARNED, NT>(a, ctx, th, blockIdx.x * NT, [rz](int row) { return __ldg(rz + row); }, S);
-    col_last_cta<DMAX, NT, LEARNED>(a, ctx, S);
-}
-
-// ---------------------------------------------------------------------------
 // Residual rebuild r = y - A x'.
 // ---------------------------------------------------------------------------
 // An injected x_hat's support (list[0, shat_count)) into the support bucket
@@ -494,6 +302,9 @@ __global__ void k_support_pairs(KArgs a, int *out)
     }
 }
 
+// Threads per block of k_collect: one per column.
+template <int DMAX> struct ColBlock { static constexpr int value = DMAX <= 8 ? 256 : (DMAX <= 16 ? 128 : 64); };
+
 // Features of every learned-scorer candidate of one round (for training logs):
 // feat[e*16..], meta[e*4..] = (column, slot, analytic pass, l1 test), omega[e],
 // in ascending (column, slot) order.  Two passes over the same arithmetic:
@@ -622,7 +433,7 @@ using rl0::Resolved;
 namespace {
 
 struct GraphEntry {
-    int nrounds, dmax, indicator, profile, learned;
+    int nrounds, indicator, profile, learned;
     cudaGraphExec_t exec;
     std::vector<cudaEvent_t> events;   // profile: 4 per round + 1, boundaries of the kernel groups
 };
@@ -652,7 +463,10 @@ struct GraphCache {
     cudaStream_t capture_stream = nullptr;
 };
 
-KArgs make_args(const rl0_expander *A)
+// The kernels' argument block of an expander, built once with its workspace.
+KArgs make_args(const rl0_expander *A) { return *(const KArgs *)A->kargs; }
+
+KArgs build_args(const rl0_expander *A)
 {
     const Workspace &w = A->ws;
     KArgs a;
@@ -691,26 +505,17 @@ KArgs make_args(const rl0_expander *A)
     a.final_part = w.final_part;
     a.res_list = w.res_list;
     rl0_res_setup(A, &a);
+    rl0_l2_setup(&a);
     return a;
 }
 
-// Launches the column score (+ H_k in its last CTA).  Returns true when it is
-// the resident-code kernel, which also fills the rebuild's buckets.
-bool launch_column_score(const KArgs &a, int dmax, int indicator, int learned, cudaStream_t s)
+// Launches the column score (+ H_k in its last CTA): the resident-code kernel
+// where it applies, else the kernel that gathers from L2.  (A failed launch is
+// left for cudaGetLastError.)
+void launch_column_score(const KArgs &a, int indicator, int learned, cudaStream_t s)
 {
-    if (rl0_res_launch(a, indicator, learned, s)) return true;
-#define RL0_CS(D, I, L) launch_pdl(k_column_score<D, I, L>, rl0_div_up(a.n, ColBlock<D>::value), ColBlock<D>::value, 0, s, a)
-    if (learned) {
-        if (dmax == 8) { if (indicator) RL0_CS(8, true, true); else RL0_CS(8, false, true); }
-        else { if (indicator) RL0_CS(16, true, true); else RL0_CS(16, false, true); }
-    } else if (dmax == 8) { if (indicator) RL0_CS(8, true, false); else RL0_CS(8, false, false); }
-    else if (dmax == 16) { if (indicator) RL0_CS(16, true, false); else RL0_CS(16, false, false); }
-    else { if (indicator) RL0_CS(32, true, false); else RL0_CS(32, false, false); }
-#undef RL0_CS
-    return false;
+    if (!rl0_res_launch(a, indicator, learned, s)) rl0_l2_launch(a, indicator, learned, s);
 }
-
-int dmax_of(int d) { return d <= 8 ? 8 : (d <= 16 ? 16 : 32); }
 
 // The residual rebuild of a round (+ accept in the rebuild's last CTA).
 void launch_rebuild(const KArgs &a, cudaStream_t s)
@@ -719,9 +524,9 @@ void launch_rebuild(const KArgs &a, cudaStream_t s)
 }
 
 // The kernels of one round (shared by the graph and by round_step).
-void launch_round(const KArgs &a, int dmax, int indicator, int learned, cudaStream_t s)
+void launch_round(const KArgs &a, int indicator, int learned, cudaStream_t s)
 {
-    launch_column_score(a, dmax, indicator, learned, s);   // + H_k in its last CTA
+    launch_column_score(a, indicator, learned, s);   // + H_k in its last CTA
     launch_rebuild(a, s);
 }
 
@@ -753,14 +558,12 @@ int add_kernel_node(cudaGraph_t g, cudaGraphNode_t *node, const cudaGraphNode_t 
     return RL0_OK;
 }
 
-int capture_decode_graph(rl0_expander *A, int nrounds, int dmax, int indicator, int profile, int learned,
-                         GraphEntry *E)
+int capture_decode_graph(rl0_expander *A, int nrounds, int indicator, int profile, int learned, GraphEntry *E)
 {
     GraphCache *gc = (GraphCache *)A->graph_cache;
     KArgs a = make_args(A);
     cudaStream_t s = gc->capture_stream;
     E->nrounds = nrounds;
-    E->dmax = dmax;
     E->indicator = indicator;
     E->profile = profile;
     E->learned = learned;
@@ -794,7 +597,7 @@ int capture_decode_graph(rl0_expander *A, int nrounds, int dmax, int indicator, 
             cudaGraph_t body = cp.conditional.phGraph_out[0];
             if (cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) !=
                 cudaSuccess) { rc = RL0_ERR_CUDA; break; }
-            for (int q = 0; q < RL0_ROUNDS_PER_ITER; ++q) launch_round(a, dmax, indicator, learned, s);
+            for (int q = 0; q < RL0_ROUNDS_PER_ITER; ++q) launch_round(a, indicator, learned, s);
             cudaGraph_t body_out = nullptr;
             if (cudaStreamEndCapture(s, &body_out) != cudaSuccess) { rc = RL0_ERR_CUDA; break; }
             // the final residual norm is taken by the step that ends the
@@ -816,7 +619,7 @@ int capture_decode_graph(rl0_expander *A, int nrounds, int dmax, int indicator, 
     cudaError_t e = cudaSuccess;
     for (int r = 0; r < nrounds && e == cudaSuccess; ++r) {
         e = mark(4 * r);
-        launch_column_score(a, dmax, indicator, learned, s);
+        launch_column_score(a, indicator, learned, s);
         if (e == cudaSuccess) e = mark(4 * r + 1);
         if (e == cudaSuccess) e = mark(4 * r + 2);
         launch_rebuild(a, s);
@@ -912,6 +715,9 @@ int rl0_workspace_alloc(rl0_expander *A)
     TableCache *tc = new (std::nothrow) TableCache;
     if (!tc) return RL0_ERR_ALLOC;
     A->table_cache = tc;
+    KArgs *ka = new (std::nothrow) KArgs(build_args(A));
+    if (!ka) return RL0_ERR_ALLOC;
+    A->kargs = ka;
     return RL0_OK;
 }
 
@@ -939,6 +745,8 @@ void rl0_workspace_free(rl0_expander *A)
         delete (TableCache *)A->table_cache;
         A->table_cache = nullptr;
     }
+    delete (KArgs *)A->kargs;
+    A->kargs = nullptr;
     void *ptrs[] = {w.rz[0], w.rz[1], w.code[0], w.code[1], w.pzlb, w.res_list, w.list, w.list_tmp, w.ulog, w.dlog, w.bcnt, w.bkt,
                     w.sbcnt[0], w.sbcnt[1], w.sbkt[0], w.sbkt[1], w.l1part, w.hk_scratch, w.st, w.ctx, w.thr, w.rlog,
                     w.final_part, w.host_y, w.host_x};
@@ -1008,17 +816,16 @@ static void cached_pz(rl0_expander *A, int64_t k, const Resolved &R, float *out)
 }
 
 // The captured round loop for this shape (captured on first use).
-static int get_graph(rl0_expander *A, int nrounds, int dmax, int indicator, int prof, int learned, GraphEntry **out)
+static int get_graph(rl0_expander *A, int nrounds, int indicator, int prof, int learned, GraphEntry **out)
 {
     GraphCache *gc = (GraphCache *)A->graph_cache;
     for (auto &g : gc->entries)
-        if (g.nrounds == nrounds && g.dmax == dmax && g.indicator == indicator && g.profile == prof &&
-            g.learned == learned) {
+        if (g.nrounds == nrounds && g.indicator == indicator && g.profile == prof && g.learned == learned) {
             *out = &g;
             return RL0_OK;
         }
     GraphEntry fresh;
-    const int rc = capture_decode_graph(A, nrounds, dmax, indicator, prof, learned, &fresh);
+    const int rc = capture_decode_graph(A, nrounds, indicator, prof, learned, &fresh);
     if (rc) {
         for (auto ev : fresh.events) if (ev) cudaEventDestroy(ev);
         return rc;
@@ -1056,13 +863,12 @@ static int launch_analytic_continuation(rl0_expander *A, const KArgs &a, int64_t
         CK(cudaMemcpyAsync((void *)a.pzlb, H->pzlb, sizeof(H->pzlb), cudaMemcpyHostToDevice, s));
     }
     CK(cudaMemsetAsync(a.st, 0, sizeof(DecodeState), s));
-    const int dmax = dmax_of(A->d);
     k_support_from_x<<<rl0_div_up(a.n, 256), 256, 0, s>>>(a);
     k_rows_from_x<<<a.nchunks, RL0_ROWS_CHUNK, 0, s>>>(a);
     k_start<<<1, 32, 0, s>>>(a, 0, 0);
     k_list_count_from_support<<<1, 32, 0, s>>>(a);
     launch_bucket_support(a, s);
-    for (int r = 0; r < R2.nrounds; ++r) launch_round(a, dmax, R2.indicator, 0, s);
+    for (int r = 0; r < R2.nrounds; ++r) launch_round(a, R2.indicator, 0, s);
     k_final_sum<<<1, 32, 0, s>>>(a);
     CK(cudaGetLastError());
     *launches = 5 + kernels_per_round(a, 0) * R2.nrounds + 1;
@@ -1079,7 +885,6 @@ static int decode_adaptive(rl0_expander *A, const float *y_dev, int64_t k, const
     HostStage *H = (HostStage *)A->host_pinned;
     const Workspace &w = A->ws;
     const KArgs a = make_args(A);
-    const int dmax = dmax_of(A->d);
     cudaEvent_t *ev = (cudaEvent_t *)A->events;
     if (stats) CK(cudaEventRecord(ev[0], s));
     k_rows_from<<<a.nchunks, RL0_ROWS_CHUNK, 0, s>>>(a, nullptr, 0, 1);
@@ -1099,7 +904,7 @@ static int decode_adaptive(rl0_expander *A, const float *y_dev, int64_t k, const
     for (int r = 0; r < H->st.round && r < RL0_MAX_ROUNDS; ++r) H->kprior[r] = kprior;   // recorded rounds
     for (int r = H->st.round; r < R.nrounds && !H->st.done; ++r) {
         H->kprior[r] = kprior;
-        launch_round(a, dmax, R.indicator, 0, s);
+        launch_round(a, R.indicator, 0, s);
         launches += kernels_per_round(a, 0);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(&H->st, w.st, sizeof(DecodeState), cudaMemcpyDeviceToHost, s));
@@ -1208,11 +1013,10 @@ static int decode_common(const rl0_expander *Ac, const float *y_dev, int64_t k, 
     CK(cudaMemsetAsync(w.st, 0, sizeof(DecodeState), s));
     if (R.p.adaptive_k) return decode_adaptive(A, y_dev, k, R, xhat_dev, stats, s);
     for (int r = 0; r < R.nrounds; ++r) H->kprior[r] = (double)k;
-    const int dmax = dmax_of(A->d);
     const int prof = R.p.profile ? 1 : 0;
     const int learned = R.p.scorer == 1;
     GraphEntry *E = nullptr;
-    rc = get_graph(A, R.nrounds, dmax, R.indicator, prof, learned, &E);
+    rc = get_graph(A, R.nrounds, R.indicator, prof, learned, &E);
     if (rc) return rc;
     cudaEvent_t *ev = (cudaEvent_t *)A->events;
     if (stats) CK(cudaEventRecord(ev[0], s));
@@ -1397,7 +1201,7 @@ extern "C" int rl0_parallel_l0(const rl0_expander *Ac, const float *y_dev, doubl
     TableCache *tc = (TableCache *)A->table_cache;
     if (tc) tc->valid = false;                     // H->ctx no longer holds a decode's cached tables
     GraphEntry *E = nullptr;
-    rc = get_graph(A, max_iter, dmax_of(A->d), 1, 0, 0, &E);
+    rc = get_graph(A, max_iter, 1, 0, 0, &E);
     if (rc) return rc;
     cudaEvent_t *ev = (cudaEvent_t *)A->events;
     if (stats) CK(cudaEventRecord(ev[0], s));
@@ -1469,7 +1273,7 @@ extern "C" int rl0_round_step(const rl0_expander *Ac, const float *y_dev, int64_
     k_start<<<1, 32, 0, s>>>(a, round_index, 0);
     k_list_count_from_support<<<1, 32, 0, s>>>(a);
     launch_bucket_support(a, s);
-    launch_round(a, dmax_of(A->d), R.indicator, R.p.scorer == 1, s);
+    launch_round(a, R.indicator, R.p.scorer == 1, s);
     k_extract_r<<<2 * a.nsm, 256, 0, s>>>(a, rp_dev, 0);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&H->st, w.st, sizeof(DecodeState), cudaMemcpyDeviceToHost, s));
@@ -1621,11 +1425,10 @@ extern "C" int rl0_decode_static(const rl0_expander *Ac, const float *y_dev, int
     CK(cudaMemsetAsync(base + L.st, 0, sizeof(DecodeState), s));
     CK(cudaMemsetAsync(base + L.bcnt, 0, sizeof(int) * (size_t)A->m, s));
 
-    const int dmax = dmax_of(A->d);
     k_rows_from<<<a.nchunks, RL0_ROWS_CHUNK, 0, s>>>(a, nullptr, 0, 1);
     k_start<<<1, 32, 0, s>>>(a, 0, 1);
     for (int r = 0; r < R.nrounds; ++r) {
-        launch_round(a, dmax, R.indicator, R.p.scorer == 1, s);
+        launch_round(a, R.indicator, R.p.scorer == 1, s);
     }
     k_final_sum<<<1, 32, 0, s>>>(a);
     CK(cudaGetLastError());

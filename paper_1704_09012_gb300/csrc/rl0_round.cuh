@@ -21,6 +21,8 @@ struct KArgs {
     int res_ok;                        // the column kernel holds every row's code in shared memory
     int res_grid;                      // its CTAs (one per SM)
     unsigned res_pz_off, res_s_off, res_q_off, res_smem;   // its dynamic shared-memory layout
+    int l2_grid[2];                    // CTAs of the L2-gather column kernel: analytic, learned (0: no variant)
+    unsigned l2_smem[2];               // its dynamic shared memory
     int res_qcap;                      // survivors per CTA staged in shared memory (FP32 residuals and x_j)
     int *res_list;                     // its other survivors: n entries of (j, candidate mask, DMAX row ids);
                                        // CTA b uses its column range
@@ -111,72 +113,6 @@ __device__ __forceinline__ void bucket_column(const KArgs &a, int j, const int *
     bucket_store<DM>(a, j, rid, d, slot);
 }
 
-// Column j's outcome: x_j += omega of its chosen anchor (best >= 0), with the
-// undo log, the support list and the nonzero count kept in step.  Every lane
-// of the warp calls it; the warp's leader takes its undo-log and list slots
-// with one atomic (take_upd_list).
-__device__ __forceinline__ void commit_column(const KArgs &a, const DecodeCtx *ctx, int j, bool active, int best,
-                                              float bw)
-{
-    const bool pass = best >= 0;
-    float old = 0.0f, nv = 0.0f;
-    if (pass) {
-        float *x = ctx->x;
-        old = x[j];
-        nv = old + bw;
-        x[j] = nv;
-    }
-    if (ctx->passed && active) ctx->passed[j] = pass ? 1 : 0;
-    const int lane = threadIdx.x & 31;
-    const unsigned mask = __ballot_sync(0xffffffffu, pass);
-    if (mask) {
-        const int leader = __ffs(mask) - 1;
-        const int dn = __reduce_add_sync(0xffffffffu, pass ? (int)(nv != 0.0f) - (int)(old != 0.0f) : 0);
-        const unsigned gone = __popc(__ballot_sync(0xffffffffu, pass && old != 0.0f && nv == 0.0f));
-        const bool fresh = pass && old == 0.0f && nv != 0.0f;
-        const unsigned fmask = __ballot_sync(0xffffffffu, fresh);
-        // d <= 8: a fresh column's row ids and bucket slots, before (and so in
-        // flight with) the leader's atomic below
-        int rid[8], slot[8];
-        const bool early = fresh && a.d <= 8;
-        if (early) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) rid[q] = (q < a.d) ? __ldg(a.rows_sm + (size_t)q * a.n + j) : 0;
-            bucket_slots<8>(a, rid, a.d, slot);
-        }
-        unsigned base = 0, fbase = 0;
-        if (lane == leader) {
-            if (dn) atomicAdd(&a.st->nnz_delta, dn);
-            if (gone) atomicAdd(&a.st->zeroed, gone);
-            const unsigned long long old2 = take_upd_list(a.st, (unsigned)__popc(mask), (unsigned)__popc(fmask));
-            base = (unsigned)(old2 >> 32);
-            fbase = (unsigned)old2;
-        }
-        base = __shfl_sync(0xffffffffu, base, leader);
-        fbase = __shfl_sync(0xffffffffu, fbase, leader);
-        const unsigned below = (1u << lane) - 1u;
-        if (pass) {
-            UndoEntry e;
-            e.j = j;
-            e.old = old;
-            a.ulog[base + __popc(mask & below)] = e;
-        }
-        if (early) {
-            a.list[fbase + __popc(fmask & below)] = j;
-            bucket_store<8>(a, j, rid, a.d, slot);
-        } else if (fresh) {
-            a.list[fbase + __popc(fmask & below)] = j;
-            // into the rebuild's fresh buckets, up to 8 rows at a time
-            for (int s0 = 0; s0 < a.d; s0 += 8) {
-                int rid[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) rid[q] = (s0 + q < a.d) ? __ldg(a.rows_sm + (size_t)(s0 + q) * a.n + j) : 0;
-                bucket_column<8>(a, j, rid, min(8, a.d - s0));
-            }
-        }
-    }
-}
-
 // A CTA's ticket at the end of a launch: after the block barrier, thread 0
 // adds one with release and acquire semantics at GPU scope, so the CTA's
 // writes are visible to whichever CTA draws the last ticket, and that CTA
@@ -189,26 +125,7 @@ __device__ __forceinline__ unsigned cta_ticket(unsigned *ctr)
     return old;
 }
 
-// The launch's last CTA applies H_k when |supp x'| > k (state read past L1,
-// since other CTAs updated it during this launch).  hk and suf are scratch of
-// that CTA; *last is a shared flag.
-template <int NT>
-__device__ __forceinline__ void last_cta_hk(const KArgs &a, const DecodeCtx *ctx, HkShared &hk, unsigned *suf,
-                                            int *last)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) *last = (cta_ticket(&a.st->col_done) == gridDim.x - 1u);
-    __syncthreads();
-    if (!*last) return;
-    DecodeState *stw = a.st;
-    const unsigned upd = __ldcg(&stw->upd_count);
-    const long long nnz = (long long)__ldcg(&stw->nnz) + __ldcg(&stw->nnz_delta);
-    if (threadIdx.x == 0) stw->col_done = 0u;
-    if (upd == 0 || nnz <= ctx->k || __ldcg(&stw->status) != 0) return;
-    cta_hk_select<NT>(a.list, __ldcg(&stw->list_count), ctx->x, ctx->k, a.hkkey, a.dlog, &stw->drop_count, hk, suf);
-}
-
-// The resident-code kernel's ticket: one acquire-release atomic per CTA adds 1
+// The column kernels' ticket: one acquire-release atomic per CTA adds 1
 // to the CTA count (bits 48..63 of DecodeState::tick) and the CTA's change of
 // the nonzero count plus 2^31 to bits 0..47 (at most 2^16 CTAs, so the biased
 // sum stays below 2^47), so that the last CTA learns |supp x'| = nnz0 + the
@@ -566,6 +483,10 @@ __device__ void accept_step(const KArgs &a, unsigned upd, unsigned *shu)
 // (res_ok = 0 when the codes do not fit the device's shared memory or the
 // workspace has no code buffers); rl0_res_launch launches it (the learned
 // scorer's variant when learned is set) and returns false when a.res_ok is 0.
+// rl0_l2_launch launches the kernel that gathers from L2 (rl0_column_l2.cu).
 void rl0_res_setup(const rl0_expander *A, KArgs *a);
 int rl0_res_dmax(int d);                     // slots per survivor-list entry for degree d
 bool rl0_res_launch(const KArgs &a, int indicator, int learned, cudaStream_t s);
+// rl0_l2_setup sets its launch shape.
+void rl0_l2_setup(KArgs *a);
+bool rl0_l2_launch(const KArgs &a, int indicator, int learned, cudaStream_t s);
