@@ -96,9 +96,11 @@ typedef struct {
     int     launches;          /* kernels launched by the decode (any mode)                  */
     int     analytic_rounds;   /* scorer = 1: rounds of the analytic continuation (0 if the  */
                                /* learned decode converged on its own)                       */
-    int     skipped_rounds;    /* rounds counted in `rounds` that launched no kernels: with   */
-                               /* sigma_n > 0 the round at t = 1 provably changes nothing    */
-                               /* (its anchor test needs p_z = 0) and is only recorded       */
+    int     skipped_rounds;    /* rounds counted in `rounds` that launched no kernels, since  */
+                               /* they provably change nothing and are only recorded: with   */
+                               /* sigma_n > 0 the round at t = 1 (its anchor test needs      */
+                               /* p_z = 0), and with the continuous or the noiseless scores  */
+                               /* rounds in which an unchanged r_hat lets no column pass     */
 } rl0_stats;
 
 /* Def. "Generating model", item 1: draw A with each column's support uniform

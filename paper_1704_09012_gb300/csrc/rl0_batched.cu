@@ -26,6 +26,7 @@
 
 #include "rl0_common.cuh"
 #include "rl0_device.cuh"
+#include "rl0_round.cuh"
 
 #define CK(call)                                          \
     do {                                                  \
@@ -39,6 +40,7 @@
 
 struct BatchItem {
     int n, m, d, nrounds, nchunks, indicator;
+    int look_ok, still_from, skip_t1;
     long long k;
     float alpha;
     double stop_level, stop_rel;
@@ -65,6 +67,7 @@ struct BatchResult {
 struct BatchState {
     int item, done, round, converged, status, overflow, nq;
     int accepted_rounds, hk_rounds, fallback_rounds, rounds_run, nnz_delta, acc;
+    int look, next_event;                           // looking ahead (rl0_round.cuh)
     unsigned upd, list_count, shat_count, drop_count, nnz, zeroed;
     double l1_hat, l1n, stop;
 };
@@ -162,9 +165,9 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
     __shared__ double s_parts[RL0_BATCH_MAX_CHUNKS];
     __shared__ double s_fpart[RL0_BATCH_MAX_CHUNKS];     // ||y - A x_hat||_1 chunk partials (FP32 pairs)
     __shared__ double s_fcand[RL0_BATCH_MAX_CHUNKS];     // the same for the candidate x'
-    __shared__ DF s_red2[NT];
     __shared__ HkShared s_hk;
     __shared__ RoundThr s_th;
+    __shared__ float s_look;
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int grp = tid / RL0_ROWS_CHUNK, gl = tid % RL0_ROWS_CHUNK;
@@ -209,18 +212,28 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
             S.status = bad ? RL0_ERR_INVALID_Y : 0;
             S.converged = (l1 <= S.stop);
             S.done = bad || S.converged || I.nrounds <= 0;
-            S.round = 0;
+            // sigma_n > 0: the round at t = 1 changes nothing and is only counted
+            const int first = (!S.done && I.skip_t1) ? 1 : 0;
+            if (first >= I.nrounds) S.done = 1;
+            S.round = first;
             S.upd = S.list_count = S.shat_count = S.drop_count = S.nnz = S.zeroed = 0;
             S.nnz_delta = S.overflow = 0;
             S.nq = 0;
-            S.accepted_rounds = S.hk_rounds = S.fallback_rounds = S.rounds_run = 0;
+            S.look = 0;
+            S.next_event = 0x7fffffff;
+            S.accepted_rounds = S.hk_rounds = S.fallback_rounds = 0;
+            S.rounds_run = first;
         }
         __syncthreads();
 
         while (!S.done) {
-            if (tid == 0) s_th = I.thr[S.round];
+            if (tid == 0) {
+                s_th = I.thr[S.round];
+                s_look = (!IND && S.look) ? I.thr[I.nrounds - 1].ta : s_th.ta;
+            }
             __syncthreads();
             const RoundThr th = s_th;
+            const float ta_look = s_look;               // the anchors this pass tests
             const float alpha = I.alpha;
 
             // ---- column scores.
@@ -234,7 +247,7 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
             // candidate slots exactly, highest first (score_anchor's arithmetic:
             // the first to pass is the last passing anchor in row order), and
             // commits.
-            const CodeThr2 ct2 = code_thresholds2(code_thresholds(th.ta, th.tz, IND ? th.te : I.pe.cut),
+            const CodeThr2 ct2 = code_thresholds2(code_thresholds(ta_look, th.tz, IND ? th.te : I.pe.cut),
                                                   IND ? alpha : alpha - 1e-3f);
             int nxa[DMAX], nxb[PAIRED ? DMAX : 1];
 #pragma unroll
@@ -275,7 +288,7 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
                                 nz += IND ? (fabsf(v.x) <= th.tz ? 1.0f : 0.0f) : v.y;
                             }
                         }
-                        ma = anchor_candidates<DMAX, IND>(r, d, th.ta, IND ? th.te : I.pe.cut, I.pe_b1, I.pe_c1, nz,
+                        ma = anchor_candidates<DMAX, IND>(r, d, ta_look, IND ? th.te : I.pe.cut, I.pe_b1, I.pe_c1, nz,
                                                           IND ? alpha : alpha - 1e-3f);
                     }
                     const unsigned ba = __ballot_sync(0xffffffffu, ma != 0u);
@@ -313,26 +326,38 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
                             r[s] = v.x;
                             nz += IND ? (fabsf(v.x) <= th.tz ? 1.0f : 0.0f) : v.y;
                             rhs += fabsf(v.x);
-                            if (((cm >> s) & 1u) && fabsf(v.x) >= th.ta) cand |= 1u << s;
+                            if (((cm >> s) & 1u) && fabsf(v.x) >= ta_look) cand |= 1u << s;
                         }
                     }
                     // the FP32 bound (exact near counts; continuous scores: an upper
                     // bound of each q_e) before the exact evaluation
                     if (cand)
-                        cand &= anchor_candidates<DMAX, IND>(r, d, th.ta, IND ? th.te : I.pe.cut, I.pe_b1, I.pe_c1,
+                        cand &= anchor_candidates<DMAX, IND>(r, d, ta_look, IND ? th.te : I.pe.cut, I.pe_b1, I.pe_c1,
                                                              nz, IND ? alpha : alpha - 1e-3f);
                     int best = -1;
-                    float bw = 0.0f;
+                    float bw = 0.0f, later = 0.0f;
                     while (cand) {
                         const int s = 31 - __clz(cand);
                         cand &= ~(1u << s);
                         const AnchorEval E = eval_anchor_regs<DMAX, IND>(r, d, s, th.te, I.pe);
                         if (E.lhs <= rhs && E.ne - nz >= alpha) {
+                            if (!IND) {
+                                float av = 0.0f;
+#pragma unroll
+                                for (int l = 0; l < DMAX; ++l)
+                                    if (l == s) av = fabsf(r[l]);
+                                if (av < th.ta) {       // an anchor of a later round
+                                    later = fmaxf(later, av);
+                                    continue;
+                                }
+                            }
                             best = s;
                             bw = E.w;
                             break;
                         }
                     }
+                    if (!IND && later > 0.0f)
+                        atomicMin(&S.next_event, anchor_round(I.thr, S.round, I.nrounds, later));
                     if (best >= 0) {
                         const float old = x[j];
                         const float nv = old + bw;
@@ -535,8 +560,16 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
                 S.overflow = 0;
                 S.nnz_delta = 0;
                 S.zeroed = 0;
-                S.round += 1;
-                S.rounds_run += 1;
+                // rounds known to change nothing are passed over (rl0_round.cuh)
+                int next = S.round + 1;
+                if (upd == 0) {
+                    if (S.look) next = min(max(S.next_event, next), I.nrounds);
+                    else if (S.round >= I.still_from) next = I.nrounds;
+                }
+                S.rounds_run += next - S.round;
+                S.round = next;
+                S.look = I.look_ok && (long long)upd * RL0_LOOK_SHARE <= I.k;
+                S.next_event = 0x7fffffff;
                 S.converged = (S.l1_hat <= S.stop);
                 if (S.converged || S.round >= I.nrounds) S.done = 1;
             }
@@ -763,6 +796,9 @@ extern "C" int rl0_decode_batched(int count, const rl0_expander *const *A, const
         It.nchunks = (int)rl0_div_up(X->m, RL0_ROWS_CHUNK);
         It.indicator = R[i].indicator;
         It.k = k[i];
+        It.look_ok = ctx[i].look_ok;
+        It.still_from = ctx[i].still_from;
+        It.skip_t1 = ctx[i].skip_t1;
         It.alpha = ctx[i].alpha;
         It.stop_level = ctx[i].stop_level;
         It.stop_rel = ctx[i].stop_rel;

@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<DMAX, LEARNED>::value
 #pragma unroll
     for (int s = 0; s < DMAX; ++s) nxt[s] = (s < d && lo + tid < hi) ? __ldg(a.rows_sm + (size_t)s * n + lo + tid) : 0;
     pdl_wait();                                    // the previous rebuild's r, x and state
-    const int done = st->done, cur = st->cur, round = st->round;
+    const int done = st->done, cur = st->cur, round = st->round, look = st->look;
     const unsigned nnz0 = st->nnz;
     pdl_launch_dependents();
     if (done) return;
@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<DMAX, LEARNED>::value
     if (tid == 0) {
         S.count = 0;
         S.dn = 0;
+        S.next_event = 0x7fffffff;
         if (!IND) S.pe = ctx->pe;
         if (LEARNED) M.R.nf = 0;
     }
@@ -90,6 +91,8 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<DMAX, LEARNED>::value
     const float need = LEARNED ? (IND ? ctx->learned_need : ctx->learned_need - 1e-3f) : (IND ? alpha : alpha - 1e-3f);
     const float reach = IND ? th.te : ctx->pe.cut, b1 = ctx->pe_b1, c1 = ctx->pe_c1;
     const int rule = ctx->anchor_rule;
+    float ta_look = th.ta;
+    if (!IND && !LEARNED && look) ta_look = a.thr[ctx->nrounds - 1].ta;
     int32_t *passed = ctx->passed;
     const float *xg = ctx->x;
     __syncthreads();
@@ -122,7 +125,7 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<DMAX, LEARNED>::value
                 r[s] = v[s].x;
                 if (s < d) nz += IND ? (fabsf(v[s].x) <= th.tz ? 1.0f : 0.0f) : v[s].y;
             }
-            const unsigned cm = active ? anchor_candidates<DMAX, IND>(r, d, th.ta, reach, b1, c1, nz, need) : 0u;
+            const unsigned cm = active ? anchor_candidates<DMAX, IND>(r, d, ta_look, reach, b1, c1, nz, need) : 0u;
             const unsigned m = __ballot_sync(0xffffffffu, cm != 0u);
             if (m) {
                 const int leader = __ffs(m) - 1;
@@ -157,10 +160,12 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<DMAX, LEARNED>::value
 #pragma unroll
                 for (int s = 0; s < DMAX; ++s) rid[s] = (s < d) ? __ldg(ids + s) : 0;
             };
-            resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, d, rule, alpha, passed, M.R, S, act, j, cm, old, v, rows);
+            resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, ta_look, round, d, rule, alpha, passed, M.R, S, act, j, cm,
+                                                  old, v, rows);
             head += min((unsigned)NT, cnt - head);
         }
     }
+    if (!IND && !LEARNED && tid == 0 && S.next_event != 0x7fffffff) atomicMin(&st->next_event, S.next_event);
     last_cta_hk_tick<NT>(a, ctx, M.h.hk, M.h.suf, &S.last, S.dn, nnz0);
 }
 

@@ -140,7 +140,7 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     }
     pdl_wait();                                    // the previous rebuild's r, codes, x and state
     // done, cur and round in one L2 trip (the code copy waits on cur)
-    const int done = st->done, cur = st->cur, round = st->round;
+    const int done = st->done, cur = st->cur, round = st->round, look = st->look;
     const unsigned nnz0 = st->nnz;
     pdl_launch_dependents();
     if (done) return false;
@@ -150,6 +150,7 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     if (tid == 0) {
         S.count = 0;
         S.dn = 0;
+        S.next_event = 0x7fffffff;
         S.nnz0 = nnz0;
         if (!IND) S.pe = ctx->pe;
         const unsigned code_bytes = 2u * (unsigned)rl0_code_rows(a.m);
@@ -190,7 +191,9 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
         }
         j0 = hi;
     }
-    const CodeThr ct = code_thresholds(th.ta, th.tz, IND ? th.te : S.pe.cut);
+    float ta_look = th.ta;
+    if (!IND && !LEARNED && look) ta_look = a.thr[ctx->nrounds - 1].ta;
+    const CodeThr ct = code_thresholds(ta_look, th.tz, IND ? th.te : S.pe.cut);
     // the count the code bound must allow: Alg. 2's alpha, or the learned
     // scorer's candidate threshold (the slack covers FP32 rounding of n_e)
     const float need0 = LEARNED ? ctx->learned_need : ctx->alpha;
@@ -367,8 +370,10 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
                 for (int s = 0; s < DMAX; ++s) rid[s] = (s < d) ? __ldcg(ent + 2 + s) : 0;
             }
         };
-        resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, d, rule, alpha, passed, R, S, act, j, cm, old, v, rows);
+        resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, ta_look, round, d, rule, alpha, passed, R, S, act, j, cm, old, v,
+                                              rows);
     }
+    if (!IND && !LEARNED && tid == 0 && S.next_event != 0x7fffffff) atomicMin(&st->next_event, S.next_event);
     return true;
 }
 

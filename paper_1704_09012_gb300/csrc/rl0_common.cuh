@@ -88,6 +88,8 @@ struct DecodeState {
     int accepted_rounds;
     int hk_rounds;
     int fallback_rounds;
+    int look;                 // the next round's column pass looks ahead (see rl0_round.cuh)
+    int next_event;           // looking ahead: the first later round in which a column would pass
     unsigned long long tick;  // resident-code column kernel: CTAs done (bits 48..63) and their
                               // changes of the nonzero count, each biased by 2^31 (bits 0..47)
     double l1_hat;
@@ -121,6 +123,9 @@ struct DecodeCtx {
     int want_log;
     int no_accept;            // round_step: stop after the rebuild (no accept, no undo)
     int always_accept;        // Alg. 1 (Parallel-l0): keep every iteration, stop when one changes nothing
+    int look_ok;              // continuous scores, analytic rule: rounds differ only in t_a, which falls
+                              // from round to round, so an unchanged r_hat can be looked ahead on
+    int still_from;           // rounds from this one on share every threshold (noiseless scores)
     int skip_t1;              // sigma_n > 0: the round at t = 1 provably changes nothing; record it only
     float conv_tol;           // Alg. 1: converged when every |r_i| <= conv_tol (0: Alg. 2's stop level)
     int wait_test;            // 0: the column kernel's first bounded wait makes its built-in number

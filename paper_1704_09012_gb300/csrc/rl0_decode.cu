@@ -125,6 +125,8 @@ __global__ void k_start(KArgs a, int round0, int empty_support)
     st->zeroed = 0;
     st->iters = 0;
     st->skipped = 0;
+    st->look = 0;
+    st->next_event = 0x7fffffff;
     if (!st->done && round0 == 0 && a.ctx->skip_t1) {
         // the round at t = 1 changes nothing (sigma_n > 0): record it as the
         // accept step records an empty round, and start at the next one
@@ -902,13 +904,15 @@ static int decode_adaptive(rl0_expander *A, const float *y_dev, int64_t k, const
     std::vector<float> vals;
     int launches = 2;
     for (int r = 0; r < H->st.round && r < RL0_MAX_ROUNDS; ++r) H->kprior[r] = kprior;   // recorded rounds
-    for (int r = H->st.round; r < R.nrounds && !H->st.done; ++r) {
-        H->kprior[r] = kprior;
+    while (H->st.round < R.nrounds && !H->st.done) {
+        const int r0 = H->st.round;
         launch_round(a, R.indicator, 0, s);
         launches += kernels_per_round(a, 0);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(&H->st, w.st, sizeof(DecodeState), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        // the round (and the recorded ones after it) used this prior
+        for (int r = r0; r < H->st.round && r < RL0_MAX_ROUNDS; ++r) H->kprior[r] = kprior;
         if (H->st.status) break;
         if (H->st.accepted_rounds == accepted) continue;
         accepted = H->st.accepted_rounds;

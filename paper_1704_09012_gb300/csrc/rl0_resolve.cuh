@@ -17,6 +17,7 @@ struct ColState {
     int count, last;                    // columns listed so far; scratch of the last-CTA test
     unsigned total, ubase, fbase;
     int dn;                             // this CTA's change of the nonzero count
+    int next_event;                     // looking ahead: the first later round in which a column passes
     unsigned nnz0;                      // |supp x_hat| at the round's start
 };
 
@@ -72,14 +73,17 @@ __device__ __forceinline__ unsigned cta_exclusive_scan(unsigned v, unsigned *wsu
 
 // One batch: thread t holds listed column j (when act) with its candidate
 // slots cm, x_j and the (r, p_z) of its rows in v; rows(rid) gives the column's
-// row ids.  Every thread of the CTA calls it; the scratch is free again when
+// row ids.  ta_look: the anchors to test (th.ta, or the sweep's last t_a when
+// the pass looks ahead; those below th.ta only report the round that makes
+// them anchors).  Every thread of the CTA calls it; the scratch is free again when
 // it returns.  The arithmetic is eval_anchor's, in its order.
 template <int DMAX, bool IND, int NT, bool LEARNED, class Rows>
-__device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *ctx, const RoundThr &th, int d, int rule,
-                                              float alpha, int32_t *passed, ResScratch<DMAX, NT, LEARNED> &R,
+__device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *ctx, const RoundThr &th, float ta_look,
+                                              int round, int d, int rule, float alpha, int32_t *passed, ResScratch<DMAX, NT, LEARNED> &R,
                                               ColState &S, bool act, int j, unsigned cm, float old, const float2 *v,
                                               Rows rows)
 {
+    constexpr bool LOOK = !IND && !LEARNED;
     const int tid = threadIdx.x;
     unsigned cand = 0u;
     if (act) {
@@ -91,7 +95,7 @@ __device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *c
                 rhs += fabsf(v[s].x);
                 // the bound's candidates that are anchors: a superset of the passing
                 // anchors, each then tested exactly below
-                if (((cm >> s) & 1u) && fabsf(v[s].x) >= th.ta) cand |= 1u << s;
+                if (((cm >> s) & 1u) && fabsf(v[s].x) >= (LOOK ? ta_look : th.ta)) cand |= 1u << s;
             }
             R.r[s][tid] = (s < d) ? v[s].x : 0.0f;
         }
@@ -185,9 +189,16 @@ __device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *c
     // last passing anchor in row order); with anchor_rule 1 the passing item
     // of largest n_e - n_z, ties to the lower slot (items come highest first)
     int best = -1;
-    float bw = 0.0f, bsc = 0.0f;
+    float bw = 0.0f, bsc = 0.0f, later = 0.0f;
     for (unsigned q = 0; q < nc; ++q)
         if (R.it_ok[off + q]) {
+            if (LOOK) {
+                const float av = fabsf(R.r[R.it_s[off + q]][tid]);
+                if (av < th.ta) {                  // an anchor of a later round
+                    later = fmaxf(later, av);
+                    continue;
+                }
+            }
             if (rule == 0) {
                 best = R.it_s[off + q];
                 bw = R.it_w[off + q];
@@ -199,6 +210,7 @@ __device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *c
                 bsc = R.it_sc[off + q];
             }
         }
+    if (LOOK && later > 0.0f) atomicMin(&S.next_event, anchor_round(a.thr, round, ctx->nrounds, later));
     const bool pass = best >= 0;
     float nv = old;
     if (pass) {

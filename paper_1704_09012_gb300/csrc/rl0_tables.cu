@@ -311,6 +311,10 @@ void fill_tables(int64_t m, int d, int64_t k, const Resolved &R, DecodeCtx *ctx,
         }
         thr[r] = T;
     }
+    ctx->look_ok = !R.indicator && p.scorer == 0;
+    for (int r = 1; r < nthr; ++r)
+        if (thr[r].ta > thr[r - 1].ta) ctx->look_ok = 0;
+    ctx->still_from = (p.sigma_n == 0.0) ? (p.quantised ? 1 : 0) : RL0_MAX_ROUNDS;
 }
 
 // Value of a non-negative FP16 bit pattern (0 .. 0x7c00; 0x7c00 is +inf).
