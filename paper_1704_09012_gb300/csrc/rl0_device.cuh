@@ -378,28 +378,6 @@ __device__ __forceinline__ void candidate_features(const float *rc, int stride, 
     f[15] = 0.0f;
 }
 
-// Logit of the MLP with parameters W (FP32 copies of the BF16 weights).
-__device__ __forceinline__ float mlp_logit(const float *W, const float *f)
-{
-    float h1[RL0_HID];
-#pragma unroll
-    for (int o = 0; o < RL0_HID; ++o) {
-        float acc = W[RL0_OFF_B1 + o];
-#pragma unroll
-        for (int i = 0; i < RL0_NFEAT; ++i) acc = fmaf(f[i], W[RL0_OFF_W1 + i * RL0_HID + o], acc);
-        h1[o] = fmaxf(acc, 0.0f);
-    }
-    float out = W[RL0_OFF_B3];
-#pragma unroll 4
-    for (int o = 0; o < RL0_HID; ++o) {
-        float acc = W[RL0_OFF_B2 + o];
-#pragma unroll
-        for (int i = 0; i < RL0_HID; ++i) acc = fmaf(h1[i], W[RL0_OFF_W2 + i * RL0_HID + o], acc);
-        out = fmaf(fmaxf(acc, 0.0f), W[RL0_OFF_W3 + o], out);
-    }
-    return out;
-}
-
 // Fast-path bound of Alg. 2's test for every anchor of a column held in
 // registers: the anchors (|r_i| >= ta) whose n_e can still reach n_z + need.
 // First level, both score kinds: n_e <= 1 + #{l != i : |r_i - r_l| <= reach}

@@ -5,9 +5,9 @@
 // weights train here; decodes use a BF16 copy with FP32 accumulation, on the
 // tensor cores (rl0_mma.cuh).
 //
-// The gradient is deterministic: each block of RL0_MLP_BLOCK samples writes its
-// own partial gradient (sums over its samples in index order), and a second
-// kernel adds the block partials in block order.
+// The gradient is deterministic: each CTA of the gradient kernel writes its own
+// partial (its tiles of 16 samples in index order), and a second kernel adds the
+// partials in a fixed order.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -17,14 +17,13 @@
 #include "rl0_common.cuh"
 #include "rl0_device.cuh"
 #include "rl0_mma.cuh"
+#include "rl0_round.cuh"
 
 #define CK(call)                                          \
     do {                                                  \
         cudaError_t e_ = (call);                          \
         if (e_ != cudaSuccess) return rl0_cuda_err(e_);   \
     } while (0)
-
-#define RL0_MLP_BLOCK 128
 
 // He-normal initial weights (std sqrt(2 / fan_in)), zero biases.  Normal
 // deviates by Box-Muller from a 64-bit mixing hash of (seed, index).
@@ -52,243 +51,458 @@ __global__ void k_mlp_init(unsigned long long seed, float *w)
     w[p] = (float)(z * sqrt(2.0 / fan));
 }
 
-// Per-block loss and gradient of the mean binary cross-entropy
+// Loss and gradient of the mean binary cross-entropy
 //   L = (1/N) sum_s softplus(o_s) - y_s o_s,   dL/do_s = (sigmoid(o_s) - y_s) / N,
-// on the tensor cores.  Warp w takes samples 16w .. 16w+15 of the block through
-// the forward pass (z1 = F W1 + b1, z2 = relu(z1) W2 + b2) and the backward pass
-// (D2 = relu'(z2) dL/do w3^T, D1 = relu'(z1) (D2 W2^T)) as m16n8k16 tiles,
-// keeping every activation in its accumulator fragment; then the block forms
-// dW1 = F^T D1 and dW2 = H1^T D2 (K = the block's samples) as 12 output tiles of
-// 16 x 8, and the vector terms (biases, w3) with FP32 sums in sample order.
-// Both operands of every product are FP32 split into three BF16 parts.
+// on the tensor cores, a block of RL0_MLP_BLOCK samples at a time.  Warp w takes
+// samples 16w .. 16w+15 through the forward pass (z1 = F W1 + b1, z2 = relu(z1)
+// W2 + b2) and the backward pass (D2 = relu'(z2) dL/do w3^T, D1 = relu'(z1)
+// (D2 W2^T)) as m16n8k16 products, every activation in its accumulator fragment,
+// which is the next product's A fragment.  movmatrix then transposes the
+// fragments whose samples become the contraction index, and the CTA forms
+// dW1 = F^T D1 and dW2 = H1^T D2 (K = the block's samples, in order) as 12 output
+// tiles of 16 x 8 from fragments in shared memory, and the vector terms
+// (biases, w3) with FP32 sums in sample order.  Both operands of every product
+// are FP32 split into three BF16 parts, each value once; the weights' parts come
+// as packed B fragments (k_mlp_pack, k_mlp_reduce_adam).
+//
+// What bounds it is latency: one block's chain of products, with one block per
+// SM and 32 blocks in a minibatch of 4096.  Splitting operands inside the
+// products' loops (the weights by every warp, X and D by every output tile), a
+// 4096-row minibatch took 35 us here, now 8.8 us.
+#define RL0_MLP_BLOCK 128
 #define RL0_MLP_WARPS (RL0_MLP_BLOCK / 16)
-#define RL0_MLP_LDF 20                                     // row pitch of F in shared memory
-#define RL0_MLP_LDH 36                                     // row pitch of H1, D1, H2, D2
+#define RL0_MLP_FWD_FRAGS 12                                // W1: 4 n-tiles; W2: 2 k-steps x 4 n-tiles
+#define RL0_MLP_FRAGS 20                                    // and W2^T: 2 k-steps x 4 n-tiles
+#define RL0_MLP_FRAG_WORDS (RL0_MLP_FRAGS * 3 * 64)         // two words per lane, three parts
+#define RL0_MLP_PITCH 1664                                  // floats per CTA partial
+#define RL0_MLP_LDH 36                                      // row pitch of D1, D2, H2
 
-__global__ void __launch_bounds__(RL0_MLP_WARPS * 32) k_mlp_grad_block(const float *__restrict__ w,
-                                                                        const float *__restrict__ feat,
-                                                                        const float *__restrict__ label,
-                                                                        long long N, float *__restrict__ part,
-                                                                        double *loss_part)
+// Shared memory of k_mlp_block: the vectors and the weights' fragments (all that
+// a pass without the gradient uses), then, per 16-sample
+// step, the A fragments of F^T and H1^T and the B fragments of D1 and D2.
+struct __align__(16) MlpShared {
+    double loss[RL0_MLP_WARPS];
+    float vec[3 * RL0_HID + 4];                             // b1, b2, w3, b3
+    uint2 frag[RL0_MLP_FRAGS * 3 * 32];
+    uint4 at[RL0_MLP_WARPS][3][3][32];                      // [step][F, H1 units 0-15, 16-31][part][lane]
+    uint2 bt[RL0_MLP_WARPS][8][3][32];                      // [step][D1 n-tiles 0-3, D2 n-tiles 0-3][part][lane]
+    float D1[RL0_MLP_BLOCK * RL0_MLP_LDH], D2[RL0_MLP_BLOCK * RL0_MLP_LDH], H2[RL0_MLP_BLOCK * RL0_MLP_LDH];
+    float DO[RL0_MLP_BLOCK];
+};
+static_assert(offsetof(MlpShared, frag) % 16 == 0 && offsetof(MlpShared, at) % 16 == 0, "16-byte copies");
+
+__device__ __forceinline__ unsigned transpose8x8(unsigned a)
 {
-    extern __shared__ float sm[];
-    float *W = sm;                                          // RL0_MLP_PARAMS (+3 pad)
-    float *F = W + RL0_MLP_PARAMS + 3;                      // [B][LDF]
-    float *H1 = F + RL0_MLP_BLOCK * RL0_MLP_LDF;            // [B][LDH] relu(z1)
-    float *D1 = H1 + RL0_MLP_BLOCK * RL0_MLP_LDH;           // [B][LDH] dL/dz1
-    float *H2 = D1 + RL0_MLP_BLOCK * RL0_MLP_LDH;           // [B][LDH] relu(z2)
-    float *D2 = H2 + RL0_MLP_BLOCK * RL0_MLP_LDH;           // [B][LDH] dL/dz2
-    float *DO = D2 + RL0_MLP_BLOCK * RL0_MLP_LDH;           // [B] dL/do
-    __shared__ double s_loss[RL0_MLP_BLOCK];
+    unsigned d;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+    return d;
+}
+
+// The A fragment (three parts) of X^T given X's A fragment.
+__device__ __forceinline__ void transpose_frag(const unsigned a[3][4], unsigned t[3][4])
+{
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        t[p][0] = transpose8x8(a[p][0]);
+        t[p][1] = transpose8x8(a[p][2]);
+        t[p][2] = transpose8x8(a[p][1]);
+        t[p][3] = transpose8x8(a[p][3]);
+    }
+}
+
+// The A fragment of X^T (three parts, from X's) to shared memory, and back.
+__device__ __forceinline__ void store_transposed(uint4 (*dst)[32], const unsigned a[3][4], int lane)
+{
+    unsigned t[3][4];
+    transpose_frag(a, t);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) dst[p][lane] = make_uint4(t[p][0], t[p][1], t[p][2], t[p][3]);
+}
+
+__device__ __forceinline__ void load_a(const uint4 (*src)[32], int lane, unsigned a[3][4])
+{
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const uint4 v = src[p][lane];
+        a[p][0] = v.x;
+        a[p][1] = v.y;
+        a[p][2] = v.z;
+        a[p][3] = v.w;
+    }
+}
+
+// The B fragments (K = the 16 samples) of the two n-tiles of 8 units that the A
+// fragment a (16 samples x 16 units) holds, to dst[0] and dst[1].
+__device__ __forceinline__ void store_b_pair(uint2 (*dst)[3][32], const unsigned a[3][4], int lane)
+{
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        dst[0][p][lane] = make_uint2(transpose8x8(a[p][0]), transpose8x8(a[p][1]));
+        dst[1][p][lane] = make_uint2(transpose8x8(a[p][2]), transpose8x8(a[p][3]));
+    }
+}
+
+__device__ __forceinline__ void load_b(const uint2 (*src)[32], int lane, unsigned b[3][2])
+{
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const uint2 v = src[p][lane];
+        b[p][0] = v.x;
+        b[p][1] = v.y;
+    }
+}
+
+// d += a . b with b a packed B fragment (part p of this lane at b[32 p])
+__device__ __forceinline__ void mma_split3_packed(float *d, const unsigned a[3][4], const uint2 *b)
+{
+    unsigned w[3][2];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const uint2 v = b[32 * p];
+        w[p][0] = v.x;
+        w[p][1] = v.y;
+    }
+    mma_split3x3(d, a, w);
+}
+
+// The packed fragments' 16-bit entries of entry (k, n) of fragment f's 16 x 8 tile.
+__device__ __forceinline__ void frag_store(unsigned short *frag, int f, int k, int n, const __nv_bfloat16 *part)
+{
+    const int reg = (k & 15) >> 3, q = (k & 7) >> 1, lane = 4 * n + q;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+        frag[(((f * 3 + p) * 32 + lane) * 2 + reg) * 2 + (k & 1)] = __bfloat16_as_ushort(part[p]);
+}
+
+// Parameter p's value v into the packed fragments.
+__device__ __forceinline__ void pack_param(unsigned short *frag, int p, float v)
+{
+    __nv_bfloat16 part[3];
+    if (p < RL0_OFF_B1) {
+        const int k = p / RL0_HID, n = p % RL0_HID;
+        split3(v, part);
+        frag_store(frag, n >> 3, k, n & 7, part);
+    } else if (p >= RL0_OFF_W2 && p < RL0_OFF_B2) {
+        const int i = (p - RL0_OFF_W2) / RL0_HID, o = (p - RL0_OFF_W2) % RL0_HID;
+        split3(v, part);
+        frag_store(frag, 4 + (i >> 4) * 4 + (o >> 3), i & 15, o & 7, part);
+        frag_store(frag, 12 + (o >> 4) * 4 + (i >> 3), o & 15, i & 7, part);     // W2^T
+    }
+}
+
+__global__ void k_mlp_pack(const float *w, unsigned short *frag)
+{
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < RL0_MLP_PARAMS) pack_param(frag, p, w[p]);
+}
+
+// GRAD: part[CTA][p] = sum of dL/dw_p over the CTA's blocks (block b to CTA
+// b mod gridDim, added in order); LOSS: loss_part[CTA] = the sum of its samples'
+// losses in FP64.  vec: feat is 8-byte aligned.
+template <bool GRAD, bool LOSS>
+__global__ void __launch_bounds__(RL0_MLP_WARPS * 32) k_mlp_block(const float *__restrict__ w,
+                                                                  const unsigned *__restrict__ frag,
+                                                                  const float *__restrict__ feat,
+                                                                  const float *__restrict__ label, long long N, int vec,
+                                                                  float *__restrict__ part, double *loss_part)
+{
+    constexpr int NF = GRAD ? RL0_MLP_FRAGS : RL0_MLP_FWD_FRAGS;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    MlpShared &M = *(MlpShared *)dsm;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const int g = lane >> 2, q = lane & 3;
-    const long long s0 = (long long)blockIdx.x * RL0_MLP_BLOCK;
-    for (int p = t; p < RL0_MLP_PARAMS; p += blockDim.x) W[p] = w[p];
-    for (int e = t; e < RL0_MLP_BLOCK * RL0_NFEAT; e += blockDim.x) {
-        const int s = e / RL0_NFEAT, i = e % RL0_NFEAT;
-        F[s * RL0_MLP_LDF + i] = (s0 + s < N) ? feat[s0 * RL0_NFEAT + e] : 0.0f;
-    }
-    __syncthreads();
-    const int r0 = 16 * wid;                                // this warp's first sample in the block
-    // ---- forward ----
-    unsigned af[3][4];
-    a_frag_split3_fn([&](int r, int c) { return F[(r0 + r) * RL0_MLP_LDF + c]; }, af);
-    float c1[4][4];
+    const long long nblocks = (N + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK;
+    // features (A fragment positions) and labels of this warp's rows g and g + 8 of block b
+    float fv[8], yl = 0.0f, yh = 0.0f;
+    auto load_block = [&](long long b) {
+        const long long sl = b * RL0_MLP_BLOCK + 16 * wid + g, sh = sl + 8;
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const float b0 = W[RL0_OFF_B1 + 8 * nt + 2 * q], b1 = W[RL0_OFF_B1 + 8 * nt + 2 * q + 1];
-        c1[nt][0] = b0;
-        c1[nt][1] = b1;
-        c1[nt][2] = b0;
-        c1[nt][3] = b1;
-        unsigned bw[3][2];
-        b_frag_split3_fn([&](int k, int n) { return W[RL0_OFF_W1 + k * RL0_HID + 8 * nt + n]; }, bw);
-        mma_split3x3(c1[nt], af, bw);
-    }
-    float c2[4][4];
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const float b0 = W[RL0_OFF_B2 + 8 * nt + 2 * q], b1 = W[RL0_OFF_B2 + 8 * nt + 2 * q + 1];
-        c2[nt][0] = b0;
-        c2[nt][1] = b1;
-        c2[nt][2] = b0;
-        c2[nt][3] = b1;
-    }
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            v[e] = fmaxf(c1[2 * kk][e], 0.0f);
-            v[4 + e] = fmaxf(c1[2 * kk + 1][e], 0.0f);
+        for (int h = 0; h < 2; ++h) {
+            const long long s = h ? sh : sl;
+            float2 v0 = make_float2(0.0f, 0.0f), v1 = v0;
+            if (s < N) {
+                const float *src = feat + s * RL0_NFEAT + 2 * q;
+                if (vec) {
+                    v0 = __ldg((const float2 *)src);
+                    v1 = __ldg((const float2 *)(src + 8));
+                } else {
+                    v0 = make_float2(src[0], src[1]);
+                    v1 = make_float2(src[8], src[9]);
+                }
+            }
+            fv[2 * h] = v0.x;
+            fv[2 * h + 1] = v0.y;
+            fv[4 + 2 * h] = v1.x;
+            fv[5 + 2 * h] = v1.y;
         }
-        unsigned a2[3][4];
-        a_frag_split3(v, a2);
+        yl = (sl < N) ? __ldg(label + sl) : 0.0f;
+        yh = (sh < N) ? __ldg(label + sh) : 0.0f;
+    };
+    load_block(blockIdx.x);                                 // (training data: no kernel writes it)
+    pdl_wait();                                             // the previous step's weights
+    pdl_launch_dependents();
+    for (int e = t; e < NF * 3 * 16; e += blockDim.x) ((uint4 *)M.frag)[e] = __ldcg((const uint4 *)frag + e);
+    for (int e = t; e < 3 * RL0_HID + 1; e += blockDim.x)
+        M.vec[e] = __ldcg(w + (e < RL0_HID ? RL0_OFF_B1 + e : (e < 2 * RL0_HID ? RL0_OFF_B2 + e - RL0_HID
+                                                                               : RL0_OFF_W3 + e - 2 * RL0_HID)));
+    __syncthreads();
+    const uint2 *B = M.frag + lane;
+    float *P = part + (size_t)blockIdx.x * RL0_MLP_PITCH;
+    double lsum = 0.0, lp = 0.0;                            // loss: sum of max(o, 0) - y o, and prod(1 + e^-|o|) - 1
+    int lcount = 0;
+    for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
+        const long long sl = b * RL0_MLP_BLOCK + 16 * wid + g;
+        const bool vl = sl < N, vh = sl + 8 < N;
+        const float y0 = yl, y1 = yh;
+        // ---- forward
+        unsigned af[3][4];
+        a_frag_split3(fv, af);
+        if (b + gridDim.x < nblocks) load_block(b + gridDim.x);
+        float c1[4][4];
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
-            unsigned bw[3][2];
-            b_frag_split3_fn([&](int k, int n) { return W[RL0_OFF_W2 + (16 * kk + k) * RL0_HID + 8 * nt + n]; }, bw);
-            mma_split3x3(c2[nt], a2, bw);
+            const float b0 = M.vec[8 * nt + 2 * q], b1 = M.vec[8 * nt + 2 * q + 1];
+            c1[nt][0] = b0;
+            c1[nt][1] = b1;
+            c1[nt][2] = b0;
+            c1[nt][3] = b1;
+            mma_split3_packed(c1[nt], af, B + 96 * nt);
         }
-    }
-    float ol = 0.0f, oh = 0.0f;                             // rows g and g + 8
+        float c2[4][4];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const float w0 = W[RL0_OFF_W3 + 8 * nt + 2 * q], w1 = W[RL0_OFF_W3 + 8 * nt + 2 * q + 1];
-        ol = fmaf(fmaxf(c2[nt][0], 0.0f), w0, ol);
-        ol = fmaf(fmaxf(c2[nt][1], 0.0f), w1, ol);
-        oh = fmaf(fmaxf(c2[nt][2], 0.0f), w0, oh);
-        oh = fmaf(fmaxf(c2[nt][3], 0.0f), w1, oh);
-    }
-    ol += __shfl_xor_sync(0xffffffffu, ol, 1);
-    ol += __shfl_xor_sync(0xffffffffu, ol, 2);
-    oh += __shfl_xor_sync(0xffffffffu, oh, 1);
-    oh += __shfl_xor_sync(0xffffffffu, oh, 2);
-    ol += W[RL0_OFF_B3];
-    oh += W[RL0_OFF_B3];
-    // ---- loss and dL/do of rows g and g + 8 ----
-    float dl, dh;
-    {
-        const long long sl = s0 + r0 + g, sh = sl + 8;
-        const bool vl = sl < N, vh = sh < N;
-        const float yl = vl ? label[sl] : 0.0f, yh = vh ? label[sh] : 0.0f;
-        dl = vl ? (1.0f / (1.0f + expf(-ol)) - yl) / (float)N : 0.0f;
-        dh = vh ? (1.0f / (1.0f + expf(-oh)) - yh) / (float)N : 0.0f;
+        for (int nt = 0; nt < 4; ++nt) {
+            const float b0 = M.vec[RL0_HID + 8 * nt + 2 * q], b1 = M.vec[RL0_HID + 8 * nt + 2 * q + 1];
+            c2[nt][0] = b0;
+            c2[nt][1] = b1;
+            c2[nt][2] = b0;
+            c2[nt][3] = b1;
+        }
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                v[e] = fmaxf(c1[2 * kk][e], 0.0f);
+                v[4 + e] = fmaxf(c1[2 * kk + 1][e], 0.0f);
+            }
+            unsigned ah[3][4];                              // relu(z1), units 16 kk .. 16 kk + 15
+            a_frag_split3(v, ah);
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) mma_split3_packed(c2[nt], ah, B + 96 * (4 + 4 * kk + nt));
+            if (GRAD) store_transposed(M.at[wid][1 + kk], ah, lane);
+        }
+        float ol = 0.0f, oh = 0.0f;                         // rows g and g + 8
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+            const float w0 = M.vec[2 * RL0_HID + 8 * nt + 2 * q], w1 = M.vec[2 * RL0_HID + 8 * nt + 2 * q + 1];
+            ol = fmaf(fmaxf(c2[nt][0], 0.0f), w0, ol);
+            ol = fmaf(fmaxf(c2[nt][1], 0.0f), w1, ol);
+            oh = fmaf(fmaxf(c2[nt][2], 0.0f), w0, oh);
+            oh = fmaf(fmaxf(c2[nt][3], 0.0f), w1, oh);
+        }
+        ol += __shfl_xor_sync(0xffffffffu, ol, 1);
+        ol += __shfl_xor_sync(0xffffffffu, ol, 2);
+        oh += __shfl_xor_sync(0xffffffffu, oh, 1);
+        oh += __shfl_xor_sync(0xffffffffu, oh, 2);
+        ol += M.vec[3 * RL0_HID];
+        oh += M.vec[3 * RL0_HID];
+        if (LOSS) {
+            // softplus(o) = max(o, 0) + log(1 + e^-|o|); the logarithm of the product
+            // of the factors is taken once per 256 of them (below 2^256)
+            const bool mine = q == 0 ? vl : (q == 1 && vh);
+            if (mine) {
+                const double o = (double)(q == 0 ? ol : oh), y = (double)(q == 0 ? y0 : y1);
+                const double e = exp(-fabs(o));
+                lp = fma(e, 1.0 + lp, lp);
+                lsum += (o > 0.0 ? o : 0.0) - y * o;
+                if (++lcount == 256) {
+                    lsum += log1p(lp);
+                    lp = 0.0;
+                    lcount = 0;
+                }
+            }
+        }
+        if (!GRAD) continue;
+        const float dl = vl ? (1.0f / (1.0f + expf(-ol)) - y0) / (float)N : 0.0f;
+        const float dh = vh ? (1.0f / (1.0f + expf(-oh)) - y1) / (float)N : 0.0f;
+        const int r0 = 16 * wid;
         if (q == 0) {
-            const double spl = (ol > 0.0f) ? (double)ol + log1p(exp(-(double)ol)) : log1p(exp((double)ol));
-            const double sph = (oh > 0.0f) ? (double)oh + log1p(exp(-(double)oh)) : log1p(exp((double)oh));
-            s_loss[r0 + g] = vl ? spl - (double)yl * (double)ol : 0.0;
-            s_loss[r0 + g + 8] = vh ? sph - (double)yh * (double)oh : 0.0;
-            DO[r0 + g] = dl;
-            DO[r0 + g + 8] = dh;
+            M.DO[r0 + g] = dl;
+            M.DO[r0 + g + 8] = dh;
         }
+        store_transposed(M.at[wid][0], af, lane);
+        // ---- backward: D2 in c2's layout, D1 = relu'(z1) (D2 W2^T)
+        float d1[4][4];
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d1[nt][e] = 0.0f;
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {                    // K = the 32 units of z2
+            float v[8];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int nt = 2 * kk + h;
+                const float w0 = M.vec[2 * RL0_HID + 8 * nt + 2 * q], w1 = M.vec[2 * RL0_HID + 8 * nt + 2 * q + 1];
+                v[4 * h] = (c2[nt][0] > 0.0f) ? dl * w0 : 0.0f;
+                v[4 * h + 1] = (c2[nt][1] > 0.0f) ? dl * w1 : 0.0f;
+                v[4 * h + 2] = (c2[nt][2] > 0.0f) ? dh * w0 : 0.0f;
+                v[4 * h + 3] = (c2[nt][3] > 0.0f) ? dh * w1 : 0.0f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int o = (r0 + g + ((e & 2) ? 8 : 0)) * RL0_MLP_LDH + 8 * nt + 2 * q + (e & 1);
+                    M.D2[o] = v[4 * h + e];
+                    M.H2[o] = fmaxf(c2[nt][e], 0.0f);
+                }
+            }
+            unsigned ad[3][4];
+            a_frag_split3(v, ad);
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) mma_split3_packed(d1[nt], ad, B + 96 * (12 + 4 * kk + nt));
+            store_b_pair(M.bt[wid] + 4 + 2 * kk, ad, lane);
+        }
+#pragma unroll
+        for (int mm = 0; mm < 2; ++mm) {
+            float v[8];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int nt = 2 * mm + h;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    v[4 * h + e] = (c1[nt][e] > 0.0f) ? d1[nt][e] : 0.0f;
+                    M.D1[(r0 + g + ((e & 2) ? 8 : 0)) * RL0_MLP_LDH + 8 * nt + 2 * q + (e & 1)] = v[4 * h + e];
+                }
+            }
+            unsigned a1[3][4];
+            a_frag_split3(v, a1);
+            store_b_pair(M.bt[wid] + 2 * mm, a1, lane);
+        }
+        __syncthreads();
+        const bool add = b != blockIdx.x;                   // a later block of this CTA
+        // ---- weight matrices: 4 tiles of dW1 (16 x 32) and 8 of dW2 (32 x 32), K = the
+        // block's samples; warps 0-3 take two of them side by side, warps 4-7 one and a vector
+        {
+            const bool two = wid < 4;
+            float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, acc2[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            const int ta = wid, tb = two ? 8 + wid : wid;   // tiles 0-3: dW1; 4-7, 8-11: dW2 units 0-15, 16-31
+#pragma unroll
+            for (int ks = 0; ks < RL0_MLP_WARPS; ++ks) {
+                unsigned a[3][4], bb[3][2];
+                load_a(M.at[ks][ta >> 2], lane, a);
+                load_b(M.bt[ks][ta < 4 ? ta : 4 + (ta & 3)], lane, bb);
+                mma_split3x3(acc, a, bb);
+                if (two) {
+                    load_a(M.at[ks][2], lane, a);
+                    load_b(M.bt[ks][4 + (tb & 3)], lane, bb);
+                    mma_split3x3(acc2, a, bb);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int row = g + ((e & 2) ? 8 : 0), c = 2 * q + (e & 1);
+                const int pa = (ta < 4 ? RL0_OFF_W1 : RL0_OFF_W2) + row * RL0_HID + 8 * (ta & 3) + c;
+                P[pa] = add ? P[pa] + acc[e] : acc[e];
+                if (two) {
+                    const int pb = RL0_OFF_W2 + (16 + row) * RL0_HID + 8 * (tb & 3) + c;
+                    P[pb] = add ? P[pb] + acc2[e] : acc2[e];
+                }
+            }
+        }
+        // ---- vectors: db1, db2, dw3 (sums over samples in index order) and db3
+        if (wid >= 4 && (wid < 7 || lane == 0)) {
+            float acc = 0.0f;
+            int po;
+            if (wid == 4) {
+                for (int s2 = 0; s2 < RL0_MLP_BLOCK; ++s2) acc += M.D1[s2 * RL0_MLP_LDH + lane];
+                po = RL0_OFF_B1 + lane;
+            } else if (wid == 5) {
+                for (int s2 = 0; s2 < RL0_MLP_BLOCK; ++s2) acc += M.D2[s2 * RL0_MLP_LDH + lane];
+                po = RL0_OFF_B2 + lane;
+            } else if (wid == 6) {
+                for (int s2 = 0; s2 < RL0_MLP_BLOCK; ++s2) acc = fmaf(M.H2[s2 * RL0_MLP_LDH + lane], M.DO[s2], acc);
+                po = RL0_OFF_W3 + lane;
+            } else {
+                for (int s2 = 0; s2 < RL0_MLP_BLOCK; ++s2) acc += M.DO[s2];
+                po = RL0_OFF_B3;
+            }
+            P[po] = add ? P[po] + acc : acc;
+        }
+        if (b + gridDim.x < nblocks) __syncthreads();       // the fragments are overwritten by the next block
     }
-    // ---- backward: D2 in c2's layout, D1 = relu'(z1) (D2 W2^T) ----
-    float d2[4][4];
+    if (LOSS) {
+        lsum += log1p(lp);
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const float w0 = W[RL0_OFF_W3 + 8 * nt + 2 * q], w1 = W[RL0_OFF_W3 + 8 * nt + 2 * q + 1];
-        d2[nt][0] = (c2[nt][0] > 0.0f) ? dl * w0 : 0.0f;
-        d2[nt][1] = (c2[nt][1] > 0.0f) ? dl * w1 : 0.0f;
-        d2[nt][2] = (c2[nt][2] > 0.0f) ? dh * w0 : 0.0f;
-        d2[nt][3] = (c2[nt][3] > 0.0f) ? dh * w1 : 0.0f;
-    }
-    float d1[4][4];
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) d1[nt][e] = 0.0f;
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {                        // K = the 32 units of z2
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            v[e] = d2[2 * kk][e];
-            v[4 + e] = d2[2 * kk + 1][e];
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        if (lane == 0) M.loss[wid] = lsum;
+        __syncthreads();
+        if (t == 0) {
+            double l = 0.0;
+            for (int v = 0; v < RL0_MLP_WARPS; ++v) l += M.loss[v];
+            loss_part[blockIdx.x] = l;
         }
-        unsigned a2[3][4];
-        a_frag_split3(v, a2);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {                    // N = the 32 units of z1; B(k, n) = W2[n][k]
-            unsigned bw[3][2];
-            b_frag_split3_fn([&](int k, int n) { return W[RL0_OFF_W2 + (8 * nt + n) * RL0_HID + 16 * kk + k]; },
-                             bw);
-            mma_split3x3(d1[nt], a2, bw);
-        }
-    }
-    // fragments to shared memory (rows r0 + g and r0 + g + 8, columns 8nt + 2q + {0, 1})
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int o = (r0 + g + ((e & 2) ? 8 : 0)) * RL0_MLP_LDH + 8 * nt + 2 * q + (e & 1);
-            H1[o] = fmaxf(c1[nt][e], 0.0f);
-            D1[o] = (c1[nt][e] > 0.0f) ? d1[nt][e] : 0.0f;
-            H2[o] = fmaxf(c2[nt][e], 0.0f);
-            D2[o] = d2[nt][e];
-        }
-    __syncthreads();
-    // ---- weight matrices: 4 tiles of dW1 (16 x 32) and 8 of dW2 (32 x 32), K = the block's samples ----
-    float *P = part + (long long)blockIdx.x * RL0_MLP_PARAMS;
-    for (int tile = wid; tile < 12; tile += RL0_MLP_WARPS) {
-        const bool l1 = tile < 4;
-        const float *X = l1 ? F : H1;                       // A = X^T
-        const float *D = l1 ? D1 : D2;                      // B = D
-        const int ldx = l1 ? RL0_MLP_LDF : RL0_MLP_LDH;
-        const int m0 = l1 ? 0 : 16 * ((tile - 4) >> 2);
-        const int n0 = 8 * (l1 ? tile : ((tile - 4) & 3));
-        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 2
-        for (int ks = 0; ks < RL0_MLP_BLOCK / 16; ++ks) {
-            unsigned ax[3][4], bd[3][2];
-            a_frag_split3_fn([&](int r, int c) { return X[(16 * ks + c) * ldx + m0 + r]; }, ax);
-            b_frag_split3_fn([&](int k, int n) { return D[(16 * ks + k) * RL0_MLP_LDH + n0 + n]; }, bd);
-            mma_split3x3(acc, ax, bd);
-        }
-        const int off = l1 ? RL0_OFF_W1 : RL0_OFF_W2;
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            P[off + (m0 + g + ((e & 2) ? 8 : 0)) * RL0_HID + n0 + 2 * q + (e & 1)] = acc[e];
-    }
-    // ---- vectors: db1, db2, dw3 (sums over samples in index order) and db3 ----
-    if (t < 3 * RL0_HID + 1) {
-        float acc = 0.0f;
-        if (t < RL0_HID) {
-            for (int s = 0; s < RL0_MLP_BLOCK; ++s) acc += D1[s * RL0_MLP_LDH + t];
-            P[RL0_OFF_B1 + t] = acc;
-        } else if (t < 2 * RL0_HID) {
-            const int o = t - RL0_HID;
-            for (int s = 0; s < RL0_MLP_BLOCK; ++s) acc += D2[s * RL0_MLP_LDH + o];
-            P[RL0_OFF_B2 + o] = acc;
-        } else if (t < 3 * RL0_HID) {
-            const int o = t - 2 * RL0_HID;
-            for (int s = 0; s < RL0_MLP_BLOCK; ++s) acc = fmaf(H2[s * RL0_MLP_LDH + o], DO[s], acc);
-            P[RL0_OFF_W3 + o] = acc;
-        } else {
-            for (int s = 0; s < RL0_MLP_BLOCK; ++s) acc += DO[s];
-            P[RL0_OFF_B3] = acc;
-        }
-    }
-    if (t == 0) {
-        double l = 0.0;
-        for (int s = 0; s < RL0_MLP_BLOCK; ++s) l += s_loss[s];
-        loss_part[blockIdx.x] = l;
     }
 }
 
-// grad[p] = sum over blocks (in block order) of the block partials.
-__global__ void k_mlp_grad_reduce(const float *part, int nblocks, float *grad, const double *loss_part, double *loss,
-                                  long long N)
+// Parameter p's gradient: the CTA partials added in CTA order, 16 loads in flight.
+#define RL0_MLP_RED 32
+__device__ __forceinline__ float sum_partials(const float *part, int nparts, int p)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < RL0_MLP_PARAMS) {
-        float acc = 0.0f;
-        for (int b = 0; b < nblocks; ++b) acc += part[(long long)b * RL0_MLP_PARAMS + p];
-        grad[p] = acc;
+    float acc = 0.0f;
+    int b = 0;
+    for (; b + 16 <= nparts; b += 16) {
+        float x[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) x[u] = __ldcg(part + (size_t)(b + u) * RL0_MLP_PITCH + p);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) acc += x[u];
     }
-    if (p == 0 && loss) {
+    for (; b < nparts; ++b) acc += __ldcg(part + (size_t)b * RL0_MLP_PITCH + p);
+    return acc;
+}
+
+// grad and the mean loss (NULL: none) from the CTA partials.
+__global__ void __launch_bounds__(RL0_MLP_RED) k_mlp_grad_reduce(const float *part, int nparts, float *grad,
+                                                                 const double *loss_part, double *loss, long long N)
+{
+    pdl_wait();
+    const int p = blockIdx.x * RL0_MLP_RED + threadIdx.x;
+    if (grad && p < RL0_MLP_PARAMS) grad[p] = sum_partials(part, nparts, p);
+    if (loss && blockIdx.x == 0) {
         double l = 0.0;
-        for (int b = 0; b < nblocks; ++b) l += loss_part[b];
-        *loss = l / (double)N;
+        for (int b = threadIdx.x; b < nparts; b += 32) l += __ldcg(loss_part + b);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (threadIdx.x == 0) *loss = l / (double)N;
     }
 }
 
-// Adam (Kingma and Ba, 2015) with bias correction, on the gradient
-// g = sum over blocks (in block order) of the block partials.
-__global__ void k_mlp_reduce_adam(const float *part, int nblocks, float *w, float *m, float *v, int step, float lr,
-                                  float b1, float b2, float eps)
+// Adam (Kingma and Ba, 2015) with bias correction on the gradient the CTA
+// partials add up to; the new weights go into the packed fragments as well.
+// One thread per parameter, its partials 16 loads at a time; the launches overlap
+// (features and moments load while the previous kernel finishes).  A 4096-row
+// step, both kernels alone (ncu): 35 + 5.4 -> 8.8 + 4.6 us; two epochs over
+// 400 003 rows with the final loss 8.66 -> 2.20 ms.
+__global__ void __launch_bounds__(RL0_MLP_RED) k_mlp_reduce_adam(const float *part, int nparts, float *w, float *m,
+                                                                 float *v, unsigned short *frag, int step, float lr,
+                                                                 float b1, float b2, float eps)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = blockIdx.x * RL0_MLP_RED + threadIdx.x;
     if (p >= RL0_MLP_PARAMS) return;
-    float gp = 0.0f;
-    for (int b = 0; b < nblocks; ++b) gp += part[(long long)b * RL0_MLP_PARAMS + p];
-    const float mp = b1 * m[p] + (1.0f - b1) * gp;
-    const float vp = b2 * v[p] + (1.0f - b2) * gp * gp;
+    // (last written two kernels ago)
+    const float m0 = __ldcg(m + p), v0 = __ldcg(v + p), w0 = __ldcg(w + p);
+    const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
+    pdl_wait();                                             // this step's partials
+    pdl_launch_dependents();
+    const float gp = sum_partials(part, nparts, p);
+    const float mp = fmaf(1.0f - b1, gp, b1 * m0);
+    const float vp = fmaf((1.0f - b2) * gp, gp, b2 * v0);
     m[p] = mp;
     v[p] = vp;
-    const float mh = mp / (1.0f - powf(b1, (float)step));
-    const float vh = vp / (1.0f - powf(b2, (float)step));
-    w[p] -= lr * mh / (sqrtf(vh) + eps);
+    const float mh = mp / c1;
+    const float vh = vp / c2;
+    const float wn = w0 - lr * mh / (sqrtf(vh) + eps);
+    w[p] = wn;
+    pack_param(frag, p, wn);
 }
 
 __global__ void k_mlp_export(const float *w, __nv_bfloat16 *wb)
@@ -317,22 +531,29 @@ __global__ void __launch_bounds__(256) k_mlp_forward(const __nv_bfloat16 *wb, co
 // ---------------------------------------------------------------------------
 // Host
 // ---------------------------------------------------------------------------
-static size_t grad_smem()
+static const unsigned kRedGrid = (RL0_MLP_PARAMS + RL0_MLP_RED - 1) / RL0_MLP_RED;
+
+static int sm_count()
 {
-    return sizeof(float) * (RL0_MLP_PARAMS + 3 + RL0_MLP_BLOCK * (RL0_MLP_LDF + 4 * RL0_MLP_LDH + 1));
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm > 0 ? nsm : 1;
 }
 
-static int mlp_grad_launch(const float *w, const float *feat, const float *label, long long N, float *grad,
-                           double *loss, float *part, double *loss_part, cudaStream_t s)
+static int mlp_blocks(long long N) { return (int)((N + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK); }
+
+// The limit on dynamic shared memory (an attribute of the kernels, set before use).
+static int mlp_smem_limit()
 {
-    const int nb = (int)((N + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK);
-    const size_t sm = grad_smem();
-    CK(cudaFuncSetAttribute((const void *)k_mlp_grad_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    k_mlp_grad_block<<<nb, RL0_MLP_WARPS * 32, sm, s>>>(w, feat, label, N, part, loss_part);
-    k_mlp_grad_reduce<<<(RL0_MLP_PARAMS + 255) / 256, 256, 0, s>>>(part, nb, grad, loss_part, loss, N);
-    CK(cudaGetLastError());
+    const int sm = (int)sizeof(MlpShared);
+    CK(cudaFuncSetAttribute((const void *)k_mlp_block<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    CK(cudaFuncSetAttribute((const void *)k_mlp_block<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    CK(cudaFuncSetAttribute((const void *)k_mlp_block<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
     return RL0_OK;
 }
+
+static int aligned8(const float *p) { return ((size_t)p & 7u) == 0; }
 
 extern "C" int rl0_mlp_init(uint64_t seed, float *w_dev, void *cuda_stream)
 {
@@ -347,18 +568,26 @@ extern "C" int rl0_mlp_grad(const float *w_dev, const float *feat_dev, const flo
 {
     if (!w_dev || !feat_dev || !label_dev || !grad_dev || N < 1) return RL0_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const int nb = (int)((N + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK);
-    float *part = nullptr;
-    double *lp = nullptr, *ld = nullptr;
-    CK(cudaMallocAsync(&part, (size_t)nb * RL0_MLP_PARAMS * sizeof(float), s));
-    CK(cudaMallocAsync(&lp, (size_t)nb * sizeof(double), s));
-    CK(cudaMallocAsync(&ld, sizeof(double), s));
-    int rc = mlp_grad_launch(w_dev, feat_dev, label_dev, N, grad_dev, ld, part, lp, s);
+    int rc = mlp_smem_limit();
+    if (rc) return rc;
+    const int grid = std::min(mlp_blocks(N), sm_count());
+    // one block: CTA partials, packed fragments, loss partials, the loss
+    const size_t o_frag = (size_t)grid * RL0_MLP_PITCH * sizeof(float);
+    const size_t o_lp = o_frag + RL0_MLP_FRAG_WORDS * sizeof(unsigned), o_ld = o_lp + (size_t)grid * sizeof(double);
+    unsigned char *buf = nullptr;
+    CK(cudaMallocAsync(&buf, o_ld + sizeof(double), s));
+    float *part = (float *)buf;
+    unsigned *frag = (unsigned *)(buf + o_frag);
+    double *lp = (double *)(buf + o_lp), *ld = (double *)(buf + o_ld);
+    k_mlp_pack<<<(RL0_MLP_PARAMS + 255) / 256, 256, 0, s>>>(w_dev, (unsigned short *)frag);
+    k_mlp_block<true, true><<<grid, RL0_MLP_WARPS * 32, sizeof(MlpShared), s>>>(w_dev, frag, feat_dev, label_dev,
+                                                                                 (long long)N, aligned8(feat_dev), part,
+                                                                                 lp);
+    k_mlp_grad_reduce<<<kRedGrid, RL0_MLP_RED, 0, s>>>(part, grid, grad_dev, lp, ld, (long long)N);
+    rc = rl0_cuda_err(cudaGetLastError());
     double l = 0.0;
     if (!rc) rc = rl0_cuda_err(cudaMemcpyAsync(&l, ld, sizeof(double), cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(part, s);
-    cudaFreeAsync(lp, s);
-    cudaFreeAsync(ld, s);
+    cudaFreeAsync(buf, s);
     if (!rc) rc = rl0_cuda_err(cudaStreamSynchronize(s));
     if (loss_host) *loss_host = l;
     return rc;
@@ -370,55 +599,55 @@ extern "C" int rl0_mlp_train(float *w_dev, const float *feat_dev, const float *l
     if (!w_dev || !feat_dev || !label_dev || N < 1 || epochs < 1 || batch < 1 || !(lr > 0.0f))
         return RL0_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const int nbmax = (batch + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK;
-    float *part = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
-    double *lp = nullptr, *ld = nullptr;
-    CK(cudaMallocAsync(&part, (size_t)nbmax * RL0_MLP_PARAMS * sizeof(float), s));
-    CK(cudaMallocAsync(&lp, (size_t)nbmax * sizeof(double), s));
-    CK(cudaMallocAsync(&ld, sizeof(double), s));
-    CK(cudaMallocAsync(&grad, RL0_MLP_PARAMS * sizeof(float), s));
-    CK(cudaMallocAsync(&m, RL0_MLP_PARAMS * sizeof(float), s));
-    CK(cudaMallocAsync(&v, RL0_MLP_PARAMS * sizeof(float), s));
-    CK(cudaMemsetAsync(m, 0, RL0_MLP_PARAMS * sizeof(float), s));
-    CK(cudaMemsetAsync(v, 0, RL0_MLP_PARAMS * sizeof(float), s));
-    int rc = RL0_OK, step = 0;
-    const size_t sm = grad_smem();
-    CK(cudaFuncSetAttribute((const void *)k_mlp_grad_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    int rc = mlp_smem_limit();
+    if (rc) return rc;
+    // a minibatch: one block per CTA; the final loss: resident CTAs (no gradient: the
+    // weights' fragments are all the shared memory they use)
+    const int gmax = mlp_blocks(std::min<int64_t>(N, batch)), gall = std::min(mlp_blocks(N), 4 * sm_count());
+    // one block: CTA partials, packed fragments, Adam's moments, loss partials, the loss
+    const size_t o_frag = (size_t)gmax * RL0_MLP_PITCH * sizeof(float);
+    const size_t o_m = o_frag + RL0_MLP_FRAG_WORDS * sizeof(unsigned), o_v = o_m + RL0_MLP_PITCH * sizeof(float);
+    const size_t o_lp = o_v + RL0_MLP_PITCH * sizeof(float), o_ld = o_lp + (size_t)gall * sizeof(double);
+    unsigned char *buf = nullptr;
+    CK(cudaMallocAsync(&buf, o_ld + sizeof(double), s));
+    float *part = (float *)buf, *m = (float *)(buf + o_m), *v = (float *)(buf + o_v);
+    unsigned *frag = (unsigned *)(buf + o_frag);
+    double *lp = (double *)(buf + o_lp), *ld = (double *)(buf + o_ld);
+    const int vec = aligned8(feat_dev);
+    rc = rl0_cuda_err(cudaMemsetAsync(m, 0, 2 * RL0_MLP_PITCH * sizeof(float), s));
+    int step = 0;
+    if (!rc) {
+        k_mlp_pack<<<(RL0_MLP_PARAMS + 255) / 256, 256, 0, s>>>(w_dev, (unsigned short *)frag);
+        rc = rl0_cuda_err(cudaGetLastError());
+    }
     for (int ep = 0; ep < epochs && !rc; ++ep) {
         for (int64_t b0 = 0; b0 < N && !rc; b0 += batch) {
             const long long nb = (N - b0 < batch) ? (N - b0) : batch;
-            const int nblk = (int)((nb + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK);
-            k_mlp_grad_block<<<nblk, RL0_MLP_WARPS * 32, sm, s>>>(w_dev, feat_dev + b0 * RL0_NFEAT, label_dev + b0,
-                                                                 nb, part, lp);
+            const int grid = mlp_blocks(nb);
+            launch_pdl(k_mlp_block<true, false>, grid, RL0_MLP_WARPS * 32, sizeof(MlpShared), s, (const float *)w_dev,
+                       (const unsigned *)frag, feat_dev + b0 * RL0_NFEAT, label_dev + b0, nb, vec, part,
+                       (double *)nullptr);
             ++step;
-            k_mlp_reduce_adam<<<(RL0_MLP_PARAMS + 255) / 256, 256, 0, s>>>(part, nblk, w_dev, m, v, step, lr, 0.9f,
-                                                                          0.999f, 1e-8f);
+            launch_pdl(k_mlp_reduce_adam, kRedGrid, RL0_MLP_RED, 0, s, (const float *)part, grid, w_dev, m, v,
+                       (unsigned short *)frag, step, lr, 0.9f, 0.999f, 1e-8f);
             rc = rl0_cuda_err(cudaGetLastError());
         }
     }
     if (!rc) {
         // loss of the final weights over the whole set
-        float *pf = nullptr;
-        double *pl = nullptr;
-        const int nball = (int)((N + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK);
-        rc = rl0_cuda_err(cudaMallocAsync(&pf, (size_t)nball * RL0_MLP_PARAMS * sizeof(float), s));
-        if (!rc) rc = rl0_cuda_err(cudaMallocAsync(&pl, (size_t)nball * sizeof(double), s));
-        if (!rc) rc = mlp_grad_launch(w_dev, feat_dev, label_dev, N, grad, ld, pf, pl, s);
+        launch_pdl(k_mlp_block<false, true>, gall, RL0_MLP_WARPS * 32, offsetof(MlpShared, at), s, (const float *)w_dev,
+                   (const unsigned *)frag, feat_dev, label_dev, (long long)N, vec, (float *)nullptr, lp);
+        launch_pdl(k_mlp_grad_reduce, 1u, RL0_MLP_RED, 0, s, (const float *)nullptr, gall, (float *)nullptr,
+                   (const double *)lp, ld, (long long)N);
         double l = 0.0;
+        rc = rl0_cuda_err(cudaGetLastError());
         if (!rc) rc = rl0_cuda_err(cudaMemcpyAsync(&l, ld, sizeof(double), cudaMemcpyDeviceToHost, s));
-        if (pf) cudaFreeAsync(pf, s);
-        if (pl) cudaFreeAsync(pl, s);
         if (!rc && wbf16_dev)
             k_mlp_export<<<(RL0_MLP_PARAMS + 255) / 256, 256, 0, s>>>(w_dev, (__nv_bfloat16 *)wbf16_dev);
         if (!rc) rc = rl0_cuda_err(cudaStreamSynchronize(s));
         if (loss_host) *loss_host = l;
     }
-    cudaFreeAsync(part, s);
-    cudaFreeAsync(lp, s);
-    cudaFreeAsync(ld, s);
-    cudaFreeAsync(grad, s);
-    cudaFreeAsync(m, s);
-    cudaFreeAsync(v, s);
+    cudaFreeAsync(buf, s);
     cudaStreamSynchronize(s);
     return rc;
 }
