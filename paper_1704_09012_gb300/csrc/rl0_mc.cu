@@ -4,8 +4,12 @@
 // "y_i = 0" over the rows and "y_i = y_l" over the row pairs of each column,
 // beside the sum of the posterior the decoder assigns to each sample.
 //
-// Integer histograms only (per-CTA shared-memory bins, merged with integer
-// atomics), so the counts do not depend on scheduling.
+// Integer histograms only, so the counts do not depend on scheduling.  A CTA
+// keeps C copies of each bin's counters in shared memory, lane l of a warp using
+// copy l mod C (a copy per lane for up to 192 bins: the lanes of a warp never
+// meet, where most samples fall into few bins), as 32-bit words: the samples, the
+// events, and the posteriors' 2^-32 units in their low 16 bits and the rest.  They
+// are added to the 64-bit bins in global memory before a word can overflow.
 #include <algorithm>
 #include <cmath>
 
@@ -14,67 +18,126 @@
 
 #define RL0_MC_MAX_BINS 1024
 #define RL0_MC_NT 256
+#define RL0_MC_WORDS 4                   // counters per bin
+#define RL0_MC_SMEM 98304                // shared memory per CTA: two fit an SM
 
 namespace {
 
-__device__ __forceinline__ unsigned long long fixed32(float p)
+struct McHist {
+    unsigned *sh;                        // [(bin * RL0_MC_WORDS + word) * C + copy]
+    int nbins, C, copy;
+};
+
+__device__ __forceinline__ void mc_add(const McHist &H, float a, bool event, float p)
 {
-    return __double2ull_rn((double)p * 4294967296.0);     // p in [0, 1], 2^-32 units
+    unsigned *h = H.sh + (unsigned)((int)a * RL0_MC_WORDS * H.C + H.copy);
+    // p in [0, 1]; scaling by 2^32 is exact, the conversion rounds to nearest even
+    const unsigned long long f = __float2ull_rn(p * 4294967296.0f);
+    atomicAdd(h, 1u);
+    if (event) atomicAdd(h + H.C, 1u);
+    atomicAdd(h + 2 * H.C, (unsigned)f & 0xffffu);
+    atomicAdd(h + 3 * H.C, (unsigned)(f >> 16));
 }
 
-__device__ __forceinline__ void mc_add(unsigned long long *h, float w, float inv_w, int nbins, bool event, float p)
-{
-    const float a = fabsf(w) * inv_w;
-    if (!(a < (float)nbins)) return;
-    const int b = (int)a;
-    atomicAdd(&h[3 * b], 1ull);
-    if (event) atomicAdd(&h[3 * b + 1], 1ull);
-    atomicAdd(&h[3 * b + 2], fixed32(p));
-}
-
-__device__ __forceinline__ void mc_flush(unsigned long long *sh, unsigned long long *out, int nbins)
+// The CTA's counters to global memory, and to zero.  Every thread calls it.
+__device__ __forceinline__ void mc_flush(const McHist &H, unsigned long long *out)
 {
     __syncthreads();
-    for (int b = threadIdx.x; b < 3 * nbins; b += blockDim.x)
-        if (sh[b]) atomicAdd(&out[b], sh[b]);
-}
-
-// Rows: bin |yhat_i|; event y0_i == 0; posterior p_breve_z(yhat_i).
-__global__ void __launch_bounds__(RL0_MC_NT) k_mc_rows(int m, const float *__restrict__ y0,
-                                                       const float *__restrict__ yh, Series pz, int nbins,
-                                                       float inv_w, unsigned long long *hz)
-{
-    __shared__ unsigned long long sh[3 * RL0_MC_MAX_BINS];
-    for (int b = threadIdx.x; b < 3 * nbins; b += blockDim.x) sh[b] = 0ull;
-    __syncthreads();
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        const float w = yh[i];
-        mc_add(sh, w, inv_w, nbins, y0[i] == 0.0f, series_eval(pz, w));
+    for (int b = threadIdx.x; b < H.nbins; b += blockDim.x) {
+        unsigned long long v[RL0_MC_WORDS];
+#pragma unroll
+        for (int w = 0; w < RL0_MC_WORDS; ++w) {
+            v[w] = 0ull;
+            unsigned *h = H.sh + (unsigned)((b * RL0_MC_WORDS + w) * H.C);
+            for (int c = 0; c < H.C; ++c) {
+                const int q = (c + b) & (H.C - 1);       // (C is a power of two: spread over the banks)
+                v[w] += h[q];
+                h[q] = 0u;
+            }
+        }
+        if (v[0]) {
+            atomicAdd(&out[3 * b], v[0]);
+            if (v[1]) atomicAdd(&out[3 * b + 1], v[1]);
+            atomicAdd(&out[3 * b + 2], v[2] + (v[3] << 16));
+        }
     }
-    mc_flush(sh, hz, nbins);
+    __syncthreads();
+}
+
+// Steps between flushes: a step adds at most RL0_MC_NT / C times `each` samples to
+// one copy of a bin, each at most 2^16 to a word, and a word stays below 2^32.
+__device__ __forceinline__ int mc_steps(int C, int each) { return max(1, (65536 / RL0_MC_NT * C - 1) / each); }
+
+__device__ __forceinline__ McHist mc_open(unsigned *sh, int nbins, int C)
+{
+    for (int e = threadIdx.x; e < nbins * RL0_MC_WORDS * C; e += blockDim.x) sh[e] = 0u;
+    __syncthreads();
+    return McHist{sh, nbins, C, (int)(threadIdx.x & (C - 1))};
+}
+
+// Rows: bin |yhat_i|; event y0_i == 0; posterior p_breve_z(yhat_i).  Also writes
+// (yhat_i, y0_i) side by side for the pairs' gathers.
+__global__ void __launch_bounds__(RL0_MC_NT) k_mc_rows(int m, const float *__restrict__ y0,
+                                                       const float *__restrict__ yh, float2 *__restrict__ both,
+                                                       Series pz, int nbins, int C, float inv_w, unsigned long long *hz)
+{
+    extern __shared__ unsigned sh[];
+    const McHist H = mc_open(sh, nbins, C);
+    const int every = mc_steps(C, 1);
+    int steps = 0;
+    for (int i0 = blockIdx.x * RL0_MC_NT; i0 < m; i0 += gridDim.x * RL0_MC_NT) {
+        const int i = i0 + threadIdx.x;
+        if (i < m) {
+            const float w = yh[i], z = y0[i];
+            both[i] = make_float2(w, z);
+            const float a = fabsf(w) * inv_w;
+            if (a < (float)nbins) mc_add(H, a, z == 0.0f, series_eval(pz, w));
+        }
+        if (++steps >= every) {
+            mc_flush(H, hz);
+            steps = 0;
+        }
+    }
+    mc_flush(H, hz);
 }
 
 // Row pairs of every column (rows ascending, s < l): bin |yhat_s - yhat_l|;
-// event y0_s == y0_l; posterior p_breve_e(yhat_s - yhat_l).
-__global__ void __launch_bounds__(RL0_MC_NT) k_mc_pairs(int n, int d, const int32_t *__restrict__ rows_cm,
-                                                        const float *__restrict__ y0, const float *__restrict__ yh,
-                                                        Series pe, int nbins, float inv_w, unsigned long long *he)
+// event y0_s == y0_l; posterior p_breve_e(yhat_s - yhat_l).  One thread per
+// column, its d values in registers (slot-major row ids: coalesced).  n = 2^20,
+// d = 7 (22 M pairs), 64 bins: 434 us with three 64-bit atomics per pair on one
+// copy of the bins -> 153 us (series and conversions, by issue).
+template <int DMAX>
+__global__ void __launch_bounds__(RL0_MC_NT) k_mc_pairs(int n, int d, const int32_t *__restrict__ rows_sm,
+                                                        const float2 *__restrict__ both, Series pe, int nbins, int C,
+                                                        float inv_w, unsigned long long *he)
 {
-    __shared__ unsigned long long sh[3 * RL0_MC_MAX_BINS];
-    for (int b = threadIdx.x; b < 3 * nbins; b += blockDim.x) sh[b] = 0ull;
-    __syncthreads();
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const int32_t *N = rows_cm + (size_t)j * d;
-        for (int s = 0; s < d; ++s) {
-            const int is = N[s];
-            for (int l = s + 1; l < d; ++l) {
-                const int il = N[l];
-                const float D = yh[is] - yh[il];
-                mc_add(sh, D, inv_w, nbins, y0[is] == y0[il], series_eval(pe, D));
+    extern __shared__ unsigned sh[];
+    const McHist H = mc_open(sh, nbins, C);
+    const int every = mc_steps(C, max(1, d * (d - 1) / 2));
+    int steps = 0;
+    for (int j0 = blockIdx.x * RL0_MC_NT; j0 < n; j0 += gridDim.x * RL0_MC_NT) {
+        const int j = j0 + threadIdx.x;
+        if (j < n) {
+            float2 v[DMAX];
+#pragma unroll
+            for (int s = 0; s < DMAX; ++s)
+                v[s] = (s < d) ? __ldg(both + __ldg(rows_sm + (size_t)s * n + j)) : make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int s = 0; s < DMAX; ++s) {
+#pragma unroll
+                for (int l = s + 1; l < DMAX; ++l) {
+                    const float D = v[s].x - v[l].x;
+                    const float a = fabsf(D) * inv_w;
+                    if (l < d && a < (float)nbins) mc_add(H, a, v[s].y == v[l].y, series_eval(pe, D));
+                }
             }
         }
+        if (++steps >= every) {
+            mc_flush(H, he);
+            steps = 0;
+        }
     }
-    mc_flush(sh, he, nbins);
+    mc_flush(H, he);
 }
 
 }  // namespace
@@ -98,11 +161,26 @@ extern "C" int rl0_posterior_mc(const rl0_expander *A, const float *y0_dev, cons
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, A->device);
     nsm = std::max(nsm, 1);
-    const int gr = (int)std::min<long long>(rl0_div_up(A->m, RL0_MC_NT), 4LL * nsm);
-    const int gp = (int)std::min<long long>(rl0_div_up(A->n, RL0_MC_NT), 4LL * nsm);
-    k_mc_rows<<<gr, RL0_MC_NT, 0, s>>>((int)A->m, y0_dev, yhat_dev, pz, nbins, (float)(nbins / wz_max),
-                                        (unsigned long long *)hz_dev);
-    k_mc_pairs<<<gp, RL0_MC_NT, 0, s>>>((int)A->n, A->d, A->rows_cm, y0_dev, yhat_dev, pe, nbins,
-                                         (float)(nbins / we_max), (unsigned long long *)he_dev);
+    int C = 32;
+    while (nbins * RL0_MC_WORDS * 4 * C > RL0_MC_SMEM) C /= 2;   // (C >= 4: nbins <= 1024)
+    const int smem = nbins * RL0_MC_WORDS * 4 * C;
+    const long long ctas = (long long)nsm * std::min(8, 2 * RL0_MC_SMEM / smem);
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if ((rc = rl0_cuda_err(cudaFuncSetAttribute(k_mc_rows, at, RL0_MC_SMEM)))) return rc;
+    // (yhat, y0) of every row side by side: the workspace is free between decodes
+    float2 *both = A->ws.rz[0];
+    const int gr = (int)std::min<long long>(rl0_div_up(A->m, RL0_MC_NT), ctas);
+    const int gp = (int)std::min<long long>(rl0_div_up(A->n, RL0_MC_NT), ctas);
+    k_mc_rows<<<gr, RL0_MC_NT, smem, s>>>((int)A->m, y0_dev, yhat_dev, both, pz, nbins, C, (float)(nbins / wz_max),
+                                          (unsigned long long *)hz_dev);
+#define RL0_MP(D) do {                                                                                              \
+        if ((rc = rl0_cuda_err(cudaFuncSetAttribute(k_mc_pairs<D>, at, RL0_MC_SMEM)))) return rc;                   \
+        k_mc_pairs<D><<<gp, RL0_MC_NT, smem, s>>>((int)A->n, A->d, A->rows_sm, both, pe, nbins, C,                  \
+                                                  (float)(nbins / we_max), (unsigned long long *)he_dev);           \
+    } while (0)
+    if (A->d <= 8) RL0_MP(8);
+    else if (A->d <= 16) RL0_MP(16);
+    else RL0_MP(32);
+#undef RL0_MP
     return rl0_cuda_err(cudaGetLastError());
 }
