@@ -160,6 +160,7 @@ struct Workspace {
     RoundLog *rlog;           // per-round log, capacity RL0_MAX_ROUNDS
     double *final_part;       // FP64 residual-norm partials, one set per rz buffer (2 x chunks)
     float *host_y, *host_x;   // rl0_decode_host's device copies of y_hat (m) and x_hat (n)
+    size_t log_bytes;         // bytes from ulog on that ulog, dlog and hk_scratch take together
     int max_rounds;
 };
 
@@ -171,6 +172,7 @@ struct rl0_expander {
     int32_t *rows_sm;         // slot-major rows: rows_sm[s*n + j], int[d*n]
     int32_t *rowptr;          // CSR of A^T: int[m+1]
     int32_t *colidx;          // CSR of A^T: int[n*d], ascending within a row
+    void *arena;              // the one device allocation behind these pointers and the workspace
     Workspace ws;
     void *graph_cache;        // captured round loops
     void *host_pinned;        // pinned staging (ctx, thresholds, stats)
@@ -226,7 +228,8 @@ int rl0_expander_finish(rl0_expander *A, cudaStream_t s);
 void rl0_expander_release(rl0_expander *A);
 
 // Decode workspace (rl0_decode.cu).
-int rl0_workspace_alloc(rl0_expander *A);
+// All of an expander's device memory (one allocation), its pinned block, stream and events.
+int rl0_workspace_alloc(rl0_expander *A, cudaStream_t s);
 void rl0_workspace_free(rl0_expander *A);
 // Host tables of (k, R) for A, cached per expander (rl0_decode.cu).
 void rl0_cached_tables(rl0_expander *A, int64_t k, const rl0::Resolved &R, DecodeCtx *ctx, RoundThr *thr);

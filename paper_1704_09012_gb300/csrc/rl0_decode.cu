@@ -663,14 +663,29 @@ struct TableCache {
 // ---------------------------------------------------------------------------
 // Workspace
 // ---------------------------------------------------------------------------
-int rl0_workspace_alloc(rl0_expander *A)
+// One allocation holds everything: an expander made per call of its user's loop
+// pays for each allocation and free (25 of them took 0.9 ms at n = 2^22).
+int rl0_workspace_alloc(rl0_expander *A, cudaStream_t s)
 {
     Workspace &w = A->ws;
-    const size_t n = (size_t)A->n, m = (size_t)A->m;
+    const size_t n = (size_t)A->n, m = (size_t)A->m, nnz = n * (size_t)A->d;
     const size_t nchunks = rl0_div_up(A->m, RL0_ROWS_CHUNK);
     w.max_rounds = RL0_MAX_ROUNDS;
-    cudaError_t e = cudaSuccess;
-    auto al = [&](void **p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
+    size_t total = 0;
+    struct Part {
+        void **p;
+        size_t off;
+    } parts[40];
+    int np = 0;
+    auto al = [&](void **p, size_t bytes) {
+        parts[np++] = Part{p, total};
+        total += (bytes + 255) & ~(size_t)255;
+    };
+    al((void **)&A->rows_cm, nnz * sizeof(int32_t));
+    al((void **)&A->rows_sm, nnz * sizeof(int32_t));
+    al((void **)&A->rowptr, (m + 1) * sizeof(int32_t));
+    al((void **)&A->colidx, nnz * sizeof(int32_t));
+    al((void **)&A->dev_flag, 64);
     al((void **)&w.rz[0], m * sizeof(float2));
     al((void **)&w.rz[1], m * sizeof(float2));
     al((void **)&w.code[0], (size_t)rl0_code_rows(A->m) * sizeof(unsigned short));
@@ -679,27 +694,30 @@ int rl0_workspace_alloc(rl0_expander *A)
     al((void **)&w.res_list, n * (size_t)(rl0_res_dmax(A->d) + 2) * sizeof(int));
     al((void **)&w.list, n * sizeof(int));
     al((void **)&w.list_tmp, sizeof(int));
+    const size_t log0 = total;
     al((void **)&w.ulog, n * sizeof(UndoEntry));
     al((void **)&w.dlog, n * sizeof(UndoEntry));
-    al((void **)&w.bcnt, m * sizeof(int));
+    al((void **)&w.hk_scratch, n * sizeof(unsigned long long));
+    w.log_bytes = total - log0;
     al((void **)&w.bkt, m * RL0_BUCKET * sizeof(int));
-    al((void **)&w.sbcnt[0], m * sizeof(int));
-    al((void **)&w.sbcnt[1], m * sizeof(int));
     al((void **)&w.sbkt[0], m * RL0_BUCKET * sizeof(int));
     al((void **)&w.sbkt[1], m * RL0_BUCKET * sizeof(int));
     al((void **)&w.l1part, nchunks * sizeof(double));
-    al((void **)&w.hk_scratch, n * sizeof(unsigned long long));
-    al((void **)&w.st, sizeof(DecodeState));
     al((void **)&w.ctx, sizeof(DecodeCtx));
     al((void **)&w.thr, RL0_MAX_ROUNDS * sizeof(RoundThr));
     al((void **)&w.rlog, RL0_MAX_ROUNDS * sizeof(RoundLog));
     al((void **)&w.final_part, 2 * nchunks * sizeof(double));   // one set per rz buffer
     al((void **)&w.host_y, m * sizeof(float));
     al((void **)&w.host_x, n * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemset(w.bcnt, 0, m * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(w.sbcnt[0], 0, m * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(w.sbcnt[1], 0, m * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(w.st, 0, sizeof(DecodeState));
+    const size_t zero0 = total;                    // what starts at zero
+    al((void **)&w.bcnt, m * sizeof(int));
+    al((void **)&w.sbcnt[0], m * sizeof(int));
+    al((void **)&w.sbcnt[1], m * sizeof(int));
+    al((void **)&w.st, sizeof(DecodeState));
+    cudaError_t e = cudaMalloc(&A->arena, total);
+    if (e != cudaSuccess) { A->arena = nullptr; cudaGetLastError(); return rl0_cuda_err(e); }
+    for (int i = 0; i < np; ++i) *parts[i].p = (unsigned char *)A->arena + parts[i].off;
+    e = cudaMemsetAsync((unsigned char *)A->arena + zero0, 0, total - zero0, s);
     if (e == cudaSuccess) e = cudaMallocHost(&A->host_pinned, sizeof(HostStage));
     if (e != cudaSuccess) { cudaGetLastError(); return rl0_cuda_err(e); }
     A->host_pinned_bytes = sizeof(HostStage);
@@ -749,10 +767,6 @@ void rl0_workspace_free(rl0_expander *A)
     }
     delete (KArgs *)A->kargs;
     A->kargs = nullptr;
-    void *ptrs[] = {w.rz[0], w.rz[1], w.code[0], w.code[1], w.pzlb, w.res_list, w.list, w.list_tmp, w.ulog, w.dlog, w.bcnt, w.bkt,
-                    w.sbcnt[0], w.sbcnt[1], w.sbkt[0], w.sbkt[1], w.l1part, w.hk_scratch, w.st, w.ctx, w.thr, w.rlog,
-                    w.final_part, w.host_y, w.host_x};
-    for (void *p : ptrs) if (p) cudaFree(p);
     std::memset(&w, 0, sizeof(w));
 }
 
