@@ -637,11 +637,13 @@ int capture_decode_graph(rl0_expander *A, int nrounds, int indicator, int profil
 }
 
 // Pinned host staging: ctx, thresholds, state, final partials, log.
+// st to thr have the same layout on the device (Workspace::st, ctx, pzlb, thr), so
+// that a decode starts with one copy of them (upload_stage).
 struct HostStage {
-    DecodeCtx ctx;
-    float pzlb[RL0_PZ_BINS];
-    DecodeState st;
-    RoundThr thr[RL0_MAX_ROUNDS];
+    alignas(128) DecodeState st;
+    alignas(128) DecodeCtx ctx;
+    alignas(128) float pzlb[RL0_PZ_BINS];          // (bulk copies read it: 16-byte aligned)
+    alignas(128) RoundThr thr[RL0_MAX_ROUNDS];
     RoundLog log[RL0_MAX_ROUNDS];
     double kprior[RL0_MAX_ROUNDS];     // the posteriors' sparsity per round (adaptive_k)
 };
@@ -690,7 +692,6 @@ int rl0_workspace_alloc(rl0_expander *A, cudaStream_t s)
     al((void **)&w.rz[1], m * sizeof(float2));
     al((void **)&w.code[0], (size_t)rl0_code_rows(A->m) * sizeof(unsigned short));
     al((void **)&w.code[1], (size_t)rl0_code_rows(A->m) * sizeof(unsigned short));
-    al((void **)&w.pzlb, RL0_PZ_BINS * sizeof(float));
     al((void **)&w.res_list, n * (size_t)(rl0_res_dmax(A->d) + 2) * sizeof(int));
     al((void **)&w.list, n * sizeof(int));
     al((void **)&w.list_tmp, sizeof(int));
@@ -703,8 +704,6 @@ int rl0_workspace_alloc(rl0_expander *A, cudaStream_t s)
     al((void **)&w.sbkt[0], m * RL0_BUCKET * sizeof(int));
     al((void **)&w.sbkt[1], m * RL0_BUCKET * sizeof(int));
     al((void **)&w.l1part, nchunks * sizeof(double));
-    al((void **)&w.ctx, sizeof(DecodeCtx));
-    al((void **)&w.thr, RL0_MAX_ROUNDS * sizeof(RoundThr));
     al((void **)&w.rlog, RL0_MAX_ROUNDS * sizeof(RoundLog));
     al((void **)&w.final_part, 2 * nchunks * sizeof(double));   // one set per rz buffer
     al((void **)&w.host_y, m * sizeof(float));
@@ -713,10 +712,13 @@ int rl0_workspace_alloc(rl0_expander *A, cudaStream_t s)
     al((void **)&w.bcnt, m * sizeof(int));
     al((void **)&w.sbcnt[0], m * sizeof(int));
     al((void **)&w.sbcnt[1], m * sizeof(int));
-    al((void **)&w.st, sizeof(DecodeState));
+    al((void **)&w.st, offsetof(HostStage, thr) + RL0_MAX_ROUNDS * sizeof(RoundThr));   // st, ctx, pzlb, thr
     cudaError_t e = cudaMalloc(&A->arena, total);
     if (e != cudaSuccess) { A->arena = nullptr; cudaGetLastError(); return rl0_cuda_err(e); }
     for (int i = 0; i < np; ++i) *parts[i].p = (unsigned char *)A->arena + parts[i].off;
+    w.ctx = (DecodeCtx *)((unsigned char *)w.st + offsetof(HostStage, ctx));
+    w.pzlb = (float *)((unsigned char *)w.st + offsetof(HostStage, pzlb));
+    w.thr = (RoundThr *)((unsigned char *)w.st + offsetof(HostStage, thr));
     e = cudaMemsetAsync((unsigned char *)A->arena + zero0, 0, total - zero0, s);
     if (e == cudaSuccess) e = cudaMallocHost(&A->host_pinned, sizeof(HostStage));
     if (e != cudaSuccess) { cudaGetLastError(); return rl0_cuda_err(e); }
@@ -851,6 +853,19 @@ static int get_graph(rl0_expander *A, int nrounds, int indicator, int prof, int 
     return RL0_OK;
 }
 
+// The settings in H (ctx, pzlb, nrounds thresholds) to the device, with fresh, also
+// a zeroed decode state: one copy, where four (three and a memset) took about 2 us
+// each before the first kernel.
+static cudaError_t upload_stage(const rl0_expander *A, int nrounds, bool fresh, cudaStream_t s)
+{
+    HostStage *H = (HostStage *)A->host_pinned;
+    if (fresh) std::memset((void *)&H->st, 0, sizeof(H->st));
+    const size_t from = fresh ? 0 : offsetof(HostStage, ctx);
+    const size_t to = offsetof(HostStage, thr) + (size_t)nrounds * sizeof(RoundThr);
+    return cudaMemcpyAsync((unsigned char *)A->ws.st + from, (const unsigned char *)H + from, to - from,
+                           cudaMemcpyHostToDevice, s);
+}
+
 // Alg. 2 with the analytic scores, continued from the x_hat a learned decode
 // left (a fresh sweep): the analytic tables, the state rebuilt from x_hat, then
 // every round of the sweep launched directly, and the final residual norm.
@@ -959,11 +974,9 @@ static int decode_adaptive(rl0_expander *A, const float *y_dev, int64_t k, const
         H->ctx.stop_level = stop_level;
         H->ctx.wait_test = A->wait_test;
         H->ctx.wait_polls = A->wait_polls;
-        CK(cudaMemcpyAsync(w.ctx, &H->ctx, sizeof(DecodeCtx), cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(w.thr, H->thr, R.nrounds * sizeof(RoundThr), cudaMemcpyHostToDevice, s));
+        if (!R.indicator) rl0::pz_lower_bounds(A->m, A->d, k, R, H->pzlb, kprior);
+        CK(upload_stage(A, R.nrounds, false, s));
         if (!R.indicator) {
-            rl0::pz_lower_bounds(A->m, A->d, k, R, H->pzlb, kprior);
-            CK(cudaMemcpyAsync(w.pzlb, H->pzlb, sizeof(H->pzlb), cudaMemcpyHostToDevice, s));
             // n_z of the next round sums p_z(r_hat) under the new prior
             k_refresh_pz<<<2 * a.nsm, 256, 0, s>>>(a);
             launches += 1;
@@ -1022,13 +1035,8 @@ static int decode_common(const rl0_expander *Ac, const float *y_dev, int64_t k, 
     H->ctx.wait_test = A->wait_test;
     H->ctx.wait_polls = A->wait_polls;
     const Workspace &w = A->ws;
-    CK(cudaMemcpyAsync(w.ctx, &H->ctx, sizeof(DecodeCtx), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(w.thr, H->thr, R.nrounds * sizeof(RoundThr), cudaMemcpyHostToDevice, s));
-    if (!R.indicator) {                           // the resident-code column kernel's n_z bound
-        cached_pz(A, k, R, H->pzlb);
-        CK(cudaMemcpyAsync(w.pzlb, H->pzlb, sizeof(H->pzlb), cudaMemcpyHostToDevice, s));
-    }
-    CK(cudaMemsetAsync(w.st, 0, sizeof(DecodeState), s));
+    if (!R.indicator) cached_pz(A, k, R, H->pzlb);   // the resident-code column kernel's n_z bound
+    CK(upload_stage(A, R.nrounds, true, s));
     if (R.p.adaptive_k) return decode_adaptive(A, y_dev, k, R, xhat_dev, stats, s);
     for (int r = 0; r < R.nrounds; ++r) H->kprior[r] = (double)k;
     const int prof = R.p.profile ? 1 : 0;
@@ -1213,9 +1221,7 @@ extern "C" int rl0_parallel_l0(const rl0_expander *Ac, const float *y_dev, doubl
     H->ctx.always_accept = 1;
     H->ctx.conv_tol = (float)tol;
     const Workspace &w = A->ws;
-    CK(cudaMemcpyAsync(w.ctx, &H->ctx, sizeof(DecodeCtx), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(w.thr, H->thr, max_iter * sizeof(RoundThr), cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(w.st, 0, sizeof(DecodeState), s));
+    CK(upload_stage(A, max_iter, true, s));
     TableCache *tc = (TableCache *)A->table_cache;
     if (tc) tc->valid = false;                     // H->ctx no longer holds a decode's cached tables
     GraphEntry *E = nullptr;
