@@ -22,6 +22,7 @@
 // 0.71 -> 0.54 ms.  What is left is the gathers: an SM asks L2 for about one
 // 32-byte sector per cycle, 0.1 ms for the 29 M of a round at n = 2^22.
 #include <algorithm>
+#include <type_traits>
 
 #include "rl0_common.cuh"
 #include "rl0_device.cuh"
@@ -45,7 +46,12 @@ struct L2Shared {
             unsigned suf[NT];
         } h;
     };
-    uint2 ring[(RL0_L2_TILES + 1) * NT];   // (column, candidate slots)
+    // (column, candidate slots), with the learned scorer in one word, (column - lo) << 8
+    // | slots (n d < 2^31 and d >= 6: a CTA of at least 152 has fewer than 2^24 columns).
+    // Its three CTAs leave little of the SM's memory to L1: with 68 KB each a decode at
+    // n = 2^22, m = 419 430 took 43.8 ms, with 62 KB 32.5.  The analytic kernel has the
+    // room and not the register (4.07 ms packed, 3.86 not).
+    std::conditional_t<LEARNED, unsigned, uint2> ring[(RL0_L2_TILES + 1) * NT];
     ColState S;
 };
 
@@ -60,6 +66,7 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
     constexpr int NT = L2NT<DMAX>::value;
     constexpr unsigned QC = (RL0_L2_TILES + 1) * NT;
     static_assert((QC & (QC - 1)) == 0, "ring positions wrap by masking");
+    static_assert(DMAX <= 8, "a ring entry holds 8 candidate slots");
     extern __shared__ __align__(16) unsigned char dsm[];
     L2Shared<DMAX, NT, LEARNED> &M = *(L2Shared<DMAX, NT, LEARNED> *)dsm;
     ColState &S = M.S;
@@ -87,6 +94,7 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
         if (!IND) S.pe = ctx->pe;
         if (LEARNED) M.R.nf = 0;
     }
+    if constexpr (LEARNED) mlp_pack(M.R.mlp, (const __nv_bfloat16 *)ctx->mlp, tid, NT);   // (read after the barriers below)
     const float alpha = ctx->alpha;
     const float need = LEARNED ? (IND ? ctx->learned_need : ctx->learned_need - 1e-3f) : (IND ? alpha : alpha - 1e-3f);
     const float reach = IND ? th.te : ctx->pe.cut, b1 = ctx->pe_b1, c1 = ctx->pe_c1;
@@ -132,7 +140,11 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
                 int base = 0;
                 if (lane == leader) base = atomicAdd(&S.count, __popc(m));
                 base = __shfl_sync(0xffffffffu, base, leader);
-                if (cm) M.ring[(unsigned)(base + __popc(m & ((1u << lane) - 1u))) & (QC - 1)] = make_uint2((unsigned)j, cm);
+                if (cm) {
+                    auto &q = M.ring[(unsigned)(base + __popc(m & ((1u << lane) - 1u))) & (QC - 1)];
+                    if constexpr (LEARNED) q = ((unsigned)(j - lo) << 8) | cm;
+                    else q = make_uint2((unsigned)j, cm);
+                }
             }
             if (passed && active && !cm) passed[j] = 0;
         }
@@ -147,9 +159,14 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
             float old = 0.0f;
             float2 v[DMAX];
             if (act) {
-                const uint2 q = M.ring[e & (QC - 1)];
-                j = (int)q.x;
-                cm = q.y;
+                const auto q = M.ring[e & (QC - 1)];
+                if constexpr (LEARNED) {
+                    j = lo + (int)(q >> 8);
+                    cm = q & 0xffu;
+                } else {
+                    j = (int)q.x;
+                    cm = q.y;
+                }
                 old = __ldca(xg + j);
                 const int *ids = a.rows_cm + (size_t)j * d;
 #pragma unroll
@@ -373,7 +390,7 @@ __device__ __forceinline__ void score_tile(const KArgs &a, const DecodeCtx *ctx,
             for (int e0 = (tid >> 5) * 16; e0 < nf; e0 += (NT / 32) * 16) {
                 auto f = [&](int r, int i) { return (e0 + r < nf) ? S.c.f[i][e0 + r] : 0.0f; };
                 float lo, hi;
-                warp_mlp_logits16(f, wb, &lo, &hi);
+                warp_mlp_logits16(f, MlpGlobal{wb}, &lo, &hi);
                 if ((tid & 3) == 0) {
                     const int gr = (tid & 31) >> 2;
                     if (e0 + gr < nf) {

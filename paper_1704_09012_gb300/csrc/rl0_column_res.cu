@@ -333,7 +333,10 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     __syncthreads();                               // the stream is done: the codes' bytes become scratch
     const int count = min(S.count, hi - lo);
     ResScratch<DMAX, NT, LEARNED> &R = *(ResScratch<DMAX, NT, LEARNED> *)dsm;
-    if (LEARNED && tid == 0) R.nf = 0;              // first read after the batch's barriers
+    if constexpr (LEARNED) {                       // first read after the batch's barriers
+        if (tid == 0) R.nf = 0;
+        if (count > 0) mlp_pack(R.mlp, (const __nv_bfloat16 *)ctx->mlp, tid, NT);
+    }
     const float alpha = ctx->alpha;
     for (int b0 = 0; b0 < count; b0 += NT) {
         // one thread per listed column: its FP32 residuals

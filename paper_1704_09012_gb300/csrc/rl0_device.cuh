@@ -352,19 +352,19 @@ static_assert(RL0_OFF_B3 + 1 == RL0_MLP_PARAMS, "parameter layout");
 __device__ __forceinline__ void candidate_features(const float *rc, int stride, int d, const AnchorEval &E, float nz,
                                                    float rhs, float inv_sn, float t, float drho, float *f)
 {
-    unsigned used = 0u;
+    // each deviation into the seven smallest so far, ascending (min and max in
+    // registers; a search per rank over the column took seven times the loads)
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-        float best = RL0_DEV_CLIP;
-        int bi = -1;
+    for (int q = 0; q < 7; ++q) f[q] = RL0_DEV_CLIP;
 #pragma unroll 1
-        for (int l = 0; l < d; ++l) {
-            if ((used >> l) & 1u) continue;
-            const float v = fminf(fabsf(rc[l * stride] - E.w) * inv_sn, RL0_DEV_CLIP);
-            if (v < best) { best = v; bi = l; }
+    for (int l = 0; l < d; ++l) {
+        float v = fminf(fabsf(rc[l * stride] - E.w) * inv_sn, RL0_DEV_CLIP);
+#pragma unroll
+        for (int q = 0; q < 7; ++q) {
+            const float lo = fminf(f[q], v);
+            v = fmaxf(f[q], v);
+            f[q] = lo;
         }
-        if (bi >= 0) used |= 1u << bi;
-        f[q] = best;
     }
     const float invd = 1.0f / (float)d;
     f[7] = E.ne * invd;

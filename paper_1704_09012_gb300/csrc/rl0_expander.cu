@@ -381,7 +381,8 @@ __global__ void __launch_bounds__(RL0_CSR_ROWS_NT) k_csr_rows(int m, CsrPlan P, 
 }
 
 // The same with a global counter per row and an insertion sort per row: more
-// entries than the buckets take (n d above about 36 million).
+// entries (n d above about 36 million) or rows (m above about a million) than the
+// buckets take.
 __global__ void k_row_count(int64_t nnz, const int32_t *rows_cm, int32_t *cnt1)
 {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

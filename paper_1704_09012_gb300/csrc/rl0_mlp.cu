@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(256) k_mlp_forward(const __nv_bfloat16 *wb, co
     if (r0 >= N) return;                           // whole warps leave together
     auto f = [&](int r, int i) { return (r0 + r < N) ? feat[(r0 + r) * RL0_NFEAT + i] : 0.0f; };
     float lo, hi;
-    warp_mlp_logits16(f, wb, &lo, &hi);
+    warp_mlp_logits16(f, MlpGlobal{wb}, &lo, &hi);
     const int g = (threadIdx.x & 31) >> 2;
     if ((threadIdx.x & 3) == 0) {
         if (r0 + g < N) logit[r0 + g] = lo;

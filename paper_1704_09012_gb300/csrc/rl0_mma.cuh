@@ -85,13 +85,71 @@ __device__ __forceinline__ void mma_split3x3(float *d, const unsigned a[3][4], c
     mma_bf16_16816(d, a[0], b[0]);
 }
 
-// Logits of 16 rows with the BF16 parameters wb (layout of rl0.h: W1 16x32
-// input-major, b1, W2 32x32, b2, w3, b3).  f(r, i) gives feature i of row r
+// The network's BF16 parameters where a warp reads them: in global memory in
+// the order of rl0.h (W1 16x32 input-major, b1, W2 32x32, b2, w3, b3), ...
+struct MlpGlobal {
+    const __nv_bfloat16 *wb;
+    // B fragment of n-tile nt of layer 1 (i = nt), of k-step kk and n-tile nt of layer 2 (i = 4 + 4 kk + nt)
+    __device__ __forceinline__ void frag(int i, unsigned b[2]) const
+    {
+        if (i < 4) b_frag_bf16(wb + RL0_OFF_W1, RL0_HID, 0, 8 * i, b);
+        else b_frag_bf16(wb + RL0_OFF_W2, RL0_HID, 16 * ((i - 4) >> 2), 8 * ((i - 4) & 3), b);
+    }
+    __device__ __forceinline__ float2 pair(int off, int u) const   // units u, u + 1 of the vector at off
+    {
+        return make_float2(__bfloat162float(wb[off + u]), __bfloat162float(wb[off + u + 1]));
+    }
+    __device__ __forceinline__ float b3() const { return __bfloat162float(wb[RL0_OFF_B3]); }
+};
+
+// ... or packed once per CTA in shared memory: every lane's fragment in one
+// 8-byte word, the vectors in FP32.  From global memory a tile of 16 rows takes
+// 48 two-byte loads of four cache lines each for the fragments and 25 more.
+// Packed, and with the features' seven smallest deviations kept in registers
+// (rl0_device.cuh): learned decodes at n = 15306, d = 7 447 -> 425 us, at n = 201716,
+// d = 9 1137 -> 1039 us, at n = 2^22, d = 7 (gathers from L2) 33.5 -> 32.6 ms.
+struct MlpPacked {
+    uint2 w[12][32];
+    float2 b1[RL0_HID / 2], b2[RL0_HID / 2], w3[RL0_HID / 2];
+    float b3v;
+    __device__ __forceinline__ void frag(int i, unsigned b[2]) const
+    {
+        const uint2 v = w[i][threadIdx.x & 31];
+        b[0] = v.x;
+        b[1] = v.y;
+    }
+    __device__ __forceinline__ float2 pair(int off, int u) const
+    {
+        const float2 *p = off == RL0_OFF_B1 ? b1 : off == RL0_OFF_B2 ? b2 : w3;
+        return p[u >> 1];
+    }
+    __device__ __forceinline__ float b3() const { return b3v; }
+};
+
+// Fills P (shared) with nt threads, a multiple of 32; a barrier follows before it is read.
+__device__ __forceinline__ void mlp_pack(MlpPacked &P, const __nv_bfloat16 *wb, int tid, int nt)
+{
+    const MlpGlobal G{wb};
+    for (int i = tid >> 5; i < 12; i += nt >> 5) {
+        unsigned b[2];
+        G.frag(i, b);
+        P.w[i][tid & 31] = make_uint2(b[0], b[1]);
+    }
+    if (tid < RL0_HID / 2) {
+        P.b1[tid] = G.pair(RL0_OFF_B1, 2 * tid);
+        P.b2[tid] = G.pair(RL0_OFF_B2, 2 * tid);
+        P.w3[tid] = G.pair(RL0_OFF_W3, 2 * tid);
+    }
+    if (tid == 0) P.b3v = G.b3();
+}
+
+// Logits of 16 rows with the parameters W (MlpGlobal or MlpPacked: the same
+// arithmetic in the same order).  f(r, i) gives feature i of row r
 // (rows 0..15 of this warp's tile).  Every lane of the warp calls it; lane
 // 4g + q returns in *lo / *hi the logits of rows g and g + 8 (the same in the
 // four lanes of a quad).
-template <class FeatFn>
-__device__ __forceinline__ void warp_mlp_logits16(FeatFn f, const __nv_bfloat16 *wb, float *lo, float *hi)
+template <class FeatFn, class Params>
+__device__ __forceinline__ void warp_mlp_logits16(FeatFn f, const Params &W, float *lo, float *hi)
 {
     const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
     // layer 1: z1 = F W1 + b1 (K = 16, four n-tiles of 8 hidden units)
@@ -111,14 +169,13 @@ __device__ __forceinline__ void warp_mlp_logits16(FeatFn f, const __nv_bfloat16 
     float c1[4][4];
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-        const float b0 = __bfloat162float(wb[RL0_OFF_B1 + 8 * nt + 2 * q]);
-        const float b1 = __bfloat162float(wb[RL0_OFF_B1 + 8 * nt + 2 * q + 1]);
-        c1[nt][0] = b0;
-        c1[nt][1] = b1;
-        c1[nt][2] = b0;
-        c1[nt][3] = b1;
+        const float2 b = W.pair(RL0_OFF_B1, 8 * nt + 2 * q);
+        c1[nt][0] = b.x;
+        c1[nt][1] = b.y;
+        c1[nt][2] = b.x;
+        c1[nt][3] = b.y;
         unsigned bw[2];
-        b_frag_bf16(wb + RL0_OFF_W1, RL0_HID, 0, 8 * nt, bw);
+        W.frag(nt, bw);
 #pragma unroll
         for (int s = 0; s < 3; ++s) mma_bf16_16816(c1[nt], a1[s], bw);
     }
@@ -126,12 +183,11 @@ __device__ __forceinline__ void warp_mlp_logits16(FeatFn f, const __nv_bfloat16 
     float c2[4][4];
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-        const float b0 = __bfloat162float(wb[RL0_OFF_B2 + 8 * nt + 2 * q]);
-        const float b1 = __bfloat162float(wb[RL0_OFF_B2 + 8 * nt + 2 * q + 1]);
-        c2[nt][0] = b0;
-        c2[nt][1] = b1;
-        c2[nt][2] = b0;
-        c2[nt][3] = b1;
+        const float2 b = W.pair(RL0_OFF_B2, 8 * nt + 2 * q);
+        c2[nt][0] = b.x;
+        c2[nt][1] = b.y;
+        c2[nt][2] = b.x;
+        c2[nt][3] = b.y;
     }
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
@@ -146,7 +202,7 @@ __device__ __forceinline__ void warp_mlp_logits16(FeatFn f, const __nv_bfloat16 
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
             unsigned bw[2];
-            b_frag_bf16(wb + RL0_OFF_W2, RL0_HID, 16 * kk, 8 * nt, bw);
+            W.frag(4 + 4 * kk + nt, bw);
 #pragma unroll
             for (int s = 0; s < 3; ++s) mma_bf16_16816(c2[nt], a2[s], bw);
         }
@@ -155,18 +211,17 @@ __device__ __forceinline__ void warp_mlp_logits16(FeatFn f, const __nv_bfloat16 
     float sl = 0.0f, sh = 0.0f;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-        const float w0 = __bfloat162float(wb[RL0_OFF_W3 + 8 * nt + 2 * q]);
-        const float w1 = __bfloat162float(wb[RL0_OFF_W3 + 8 * nt + 2 * q + 1]);
-        sl = fmaf(fmaxf(c2[nt][0], 0.0f), w0, sl);
-        sl = fmaf(fmaxf(c2[nt][1], 0.0f), w1, sl);
-        sh = fmaf(fmaxf(c2[nt][2], 0.0f), w0, sh);
-        sh = fmaf(fmaxf(c2[nt][3], 0.0f), w1, sh);
+        const float2 w = W.pair(RL0_OFF_W3, 8 * nt + 2 * q);
+        sl = fmaf(fmaxf(c2[nt][0], 0.0f), w.x, sl);
+        sl = fmaf(fmaxf(c2[nt][1], 0.0f), w.y, sl);
+        sh = fmaf(fmaxf(c2[nt][2], 0.0f), w.x, sh);
+        sh = fmaf(fmaxf(c2[nt][3], 0.0f), w.y, sh);
     }
     sl += __shfl_xor_sync(0xffffffffu, sl, 1);
     sl += __shfl_xor_sync(0xffffffffu, sl, 2);
     sh += __shfl_xor_sync(0xffffffffu, sh, 1);
     sh += __shfl_xor_sync(0xffffffffu, sh, 2);
-    const float b3 = __bfloat162float(wb[RL0_OFF_B3]);
+    const float b3 = W.b3();
     *lo = sl + b3;
     *hi = sh + b3;
 }

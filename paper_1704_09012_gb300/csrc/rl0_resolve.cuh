@@ -5,6 +5,8 @@
 // kernels (rl0_column_res.cu, rl0_column_l2.cu).  Not part of the ABI.
 #pragma once
 
+#include <type_traits>
+
 #include "rl0_common.cuh"
 #include "rl0_device.cuh"
 #include "rl0_mma.cuh"
@@ -33,8 +35,12 @@ struct ResScratch {
     unsigned char it_ok[NT * DMAX];
     float it_w[NT * DMAX];
     float it_sc[NT * DMAX];              // n_e - n_z of the item
-    float feat[LEARNED ? NT : 1][RL0_NFEAT];   // learned scorer: features of the items that pass the
-    unsigned short fidx[LEARNED ? NT : 1];     // exact tests (compact, NT items at a time) and their items
+    // learned scorer: features of the items that pass the exact tests (compact, NT
+    // items at a time; by feature, the pitch keeps a tile's eight rows times four
+    // feature pairs on different banks; f14 = f15 = 0 are not held), their items, and the network
+    float feat[RL0_NFEAT - 2][LEARNED ? NT + 4 : 1];
+    unsigned short fidx[LEARNED ? NT : 1];
+    std::conditional_t<LEARNED, MlpPacked, int> mlp;
     float q[NT][DMAX];                   // q_e of (item, slot l), NT items at a time
     unsigned wsum[NT / 32];
     int nf;
@@ -157,7 +163,7 @@ __device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *c
                     candidate_features(&R.r[0][ee], NT, d, E, R.nz[ee], R.rhs[ee], ctx->inv_sn, th.t, ctx->drho, f);
                     const int p = atomicAdd(&R.nf, 1);
 #pragma unroll
-                    for (int q = 0; q < RL0_NFEAT; ++q) R.feat[p][q] = f[q];
+                    for (int q = 0; q < RL0_NFEAT - 2; ++q) R.feat[q][p] = f[q];
                     R.fidx[p] = (unsigned short)kk;
                 }
             } else {
@@ -170,11 +176,10 @@ __device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *c
         if constexpr (LEARNED) {
             // the passing items' logits, 16 per warp on the tensor cores
             const unsigned nf = (unsigned)R.nf;
-            const __nv_bfloat16 *wb = (const __nv_bfloat16 *)ctx->mlp;
             for (unsigned t0 = (unsigned)(tid >> 5) * 16u; t0 < nf; t0 += (NT / 32) * 16u) {
-                auto f = [&](int r, int i) { return (t0 + r < nf) ? R.feat[t0 + r][i] : 0.0f; };
+                auto f = [&](int r, int i) { return (t0 + r < nf && i < RL0_NFEAT - 2) ? R.feat[i][t0 + r] : 0.0f; };
                 float lo, hi;
-                warp_mlp_logits16(f, wb, &lo, &hi);
+                warp_mlp_logits16(f, R.mlp, &lo, &hi);
                 if ((tid & 3) == 0) {
                     const unsigned gr = (unsigned)((tid & 31) >> 2);
                     if (t0 + gr < nf && !(lo >= ctx->logit_thr)) R.it_ok[k0 + R.fidx[t0 + gr]] = 0;
