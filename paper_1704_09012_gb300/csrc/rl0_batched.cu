@@ -59,14 +59,14 @@ struct BatchItem {
 };
 
 struct BatchResult {
-    int rounds, accepted_rounds, converged, status, hk_rounds, fallback_rounds;
+    int rounds, accepted_rounds, converged, status, hk_rounds, fallback_rounds, skipped;
     unsigned nnz;
     double l1_hat, final_l1;
 };
 
 struct BatchState {
     int item, done, round, converged, status, overflow, nq;
-    int accepted_rounds, hk_rounds, fallback_rounds, rounds_run, nnz_delta, acc;
+    int accepted_rounds, hk_rounds, fallback_rounds, rounds_run, skipped, nnz_delta, acc;
     int look, next_event;                           // looking ahead (rl0_round.cuh)
     unsigned upd, list_count, shat_count, drop_count, nnz, zeroed;
     double l1_hat, l1n, stop;
@@ -223,6 +223,7 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
             S.next_event = 0x7fffffff;
             S.accepted_rounds = S.hk_rounds = S.fallback_rounds = 0;
             S.rounds_run = first;
+            S.skipped = first;
         }
         __syncthreads();
 
@@ -567,6 +568,7 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
                     else if (S.round >= I.still_from) next = I.nrounds;
                 }
                 S.rounds_run += next - S.round;
+                S.skipped += next - S.round - 1;
                 S.round = next;
                 S.look = I.look_ok && (long long)upd * RL0_LOOK_SHARE <= I.k;
                 S.next_event = 0x7fffffff;
@@ -589,6 +591,7 @@ __global__ void __launch_bounds__(NT, 1) k_decode_batched(const BatchItem *__res
                 R.status = S.status;
                 R.hk_rounds = S.hk_rounds;
                 R.fallback_rounds = S.fallback_rounds;
+                R.skipped = S.skipped;
                 R.nnz = S.nnz;
                 R.l1_hat = S.l1_hat;
                 R.final_l1 = fl;
@@ -900,6 +903,7 @@ extern "C" int rl0_decode_batched(int count, const rl0_expander *const *A, const
             S.ms = ms;
             S.hk_rounds = Rr.hk_rounds;
             S.fallback_rounds = Rr.fallback_rounds;
+            S.skipped_rounds = Rr.skipped;
             S.launches = (q == 0) ? 1 : 0;
         }
     }
