@@ -149,8 +149,11 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
             if (passed && active && !cm) passed[j] = 0;
         }
         __syncthreads();
-        // ---- resolve full batches (at the end, the rest too)
+        // ---- resolve full batches (at the end, the rest too).  Every thread takes the
+        // same count: the next chunk adds to it only after all have read it, also when
+        // no batch is resolved (whose barriers would keep the warps together).
         const unsigned cnt = (unsigned)S.count;
+        __syncthreads();
         while (cnt - head >= (unsigned)NT || (j0 >= hi && cnt != head)) {
             const unsigned e = head + (unsigned)tid;
             const bool act = e < cnt;
