@@ -466,7 +466,8 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value) k_column_score_tile(KArgs a
     last_cta_hk<NT>(a, ctx, S.h.hk, S.h.suf, &S.last);
 }
 
-// Launch shape of a variant: as many CTAs as the SMs hold at once.
+// Launch shape of a variant: as many CTAs as the SMs hold at once (0 when the device
+// refuses it: a decode that needs the variant returns RL0_ERR_CUDA).
 template <int DMAX, bool LEARNED>
 void l2_shape(KArgs *a)
 {
@@ -518,10 +519,10 @@ struct L2Shape {
 
 template <int DMAX, bool EXACT, bool LEARNED>
 struct L2Launch {
-    static bool call(const KArgs *a, int indicator, cudaStream_t s)
+    static int call(const KArgs *a, int indicator, cudaStream_t s)
     {
         const int grid = a->l2_grid[LEARNED];
-        if (grid < 1) return false;
+        if (grid < 1) return RL0_ERR_CUDA;          // the setup could not get the kernel's shape
         constexpr int NT = L2NT<DMAX>::value;
         const unsigned sm = a->l2_smem[LEARNED];
         if constexpr (EXACT) {
@@ -531,7 +532,7 @@ struct L2Launch {
             if (indicator) launch_pdl(k_column_score_tile<DMAX, true, LEARNED>, grid, NT, sm, s, *a);
             else launch_pdl(k_column_score_tile<DMAX, false, LEARNED>, grid, NT, sm, s, *a);
         }
-        return true;
+        return RL0_OK;
     }
 };
 
@@ -543,7 +544,7 @@ void rl0_l2_setup(KArgs *a)
     if (a->d <= 16) l2_variant<L2Shape, true>(a->d, a);
 }
 
-bool rl0_l2_launch(const KArgs &a, int indicator, int learned, cudaStream_t s)
+int rl0_l2_launch(const KArgs &a, int indicator, int learned, cudaStream_t s)
 {
     return learned ? l2_variant<L2Launch, true>(a.d, &a, indicator, s) : l2_variant<L2Launch, false>(a.d, &a, indicator, s);
 }

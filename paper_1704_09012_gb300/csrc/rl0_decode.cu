@@ -40,6 +40,11 @@
         cudaError_t e_ = (call);                          \
         if (e_ != cudaSuccess) return rl0_cuda_err(e_);   \
     } while (0)
+#define RC(call)                                          \
+    do {                                                  \
+        const int rc_ = (call);                           \
+        if (rc_) return rc_;                              \
+    } while (0)
 
 
 // r source -> rz[dst] = (r, p_z(r)), the l1 partial (FP32 pairs, stored in FP64) of each RL0_ROWS_CHUNK-row
@@ -512,11 +517,11 @@ KArgs build_args(const rl0_expander *A)
 }
 
 // Launches the column score (+ H_k in its last CTA): the resident-code kernel
-// where it applies, else the kernel that gathers from L2.  (A failed launch is
-// left for cudaGetLastError.)
-void launch_column_score(const KArgs &a, int indicator, int learned, cudaStream_t s)
+// where it applies, else the kernel that gathers from L2; an error when there is
+// neither.  (A failed launch is left for cudaGetLastError.)
+[[nodiscard]] int launch_column_score(const KArgs &a, int indicator, int learned, cudaStream_t s)
 {
-    if (!rl0_res_launch(a, indicator, learned, s)) rl0_l2_launch(a, indicator, learned, s);
+    return rl0_res_launch(a, indicator, learned, s) ? RL0_OK : rl0_l2_launch(a, indicator, learned, s);
 }
 
 // The residual rebuild of a round (+ accept in the rebuild's last CTA).
@@ -526,10 +531,11 @@ void launch_rebuild(const KArgs &a, cudaStream_t s)
 }
 
 // The kernels of one round (shared by the graph and by round_step).
-void launch_round(const KArgs &a, int indicator, int learned, cudaStream_t s)
+[[nodiscard]] int launch_round(const KArgs &a, int indicator, int learned, cudaStream_t s)
 {
-    launch_column_score(a, indicator, learned, s);   // + H_k in its last CTA
-    launch_rebuild(a, s);
+    const int rc = launch_column_score(a, indicator, learned, s);   // + H_k in its last CTA
+    if (!rc) launch_rebuild(a, s);
+    return rc;
 }
 
 // An injected x_hat's support into the support bucket B[0].
@@ -599,9 +605,10 @@ int capture_decode_graph(rl0_expander *A, int nrounds, int indicator, int profil
             cudaGraph_t body = cp.conditional.phGraph_out[0];
             if (cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) !=
                 cudaSuccess) { rc = RL0_ERR_CUDA; break; }
-            for (int q = 0; q < RL0_ROUNDS_PER_ITER; ++q) launch_round(a, indicator, learned, s);
+            for (int q = 0; q < RL0_ROUNDS_PER_ITER && !rc; ++q) rc = launch_round(a, indicator, learned, s);
             cudaGraph_t body_out = nullptr;
-            if (cudaStreamEndCapture(s, &body_out) != cudaSuccess) { rc = RL0_ERR_CUDA; break; }
+            if (cudaStreamEndCapture(s, &body_out) != cudaSuccess) rc = RL0_ERR_CUDA;
+            if (rc) break;
             // the final residual norm is taken by the step that ends the
             // decode (k_start or the accept step): no epilogue kernel
         } while (0);
@@ -619,9 +626,10 @@ int capture_decode_graph(rl0_expander *A, int nrounds, int indicator, int profil
     k_rows_from<<<a.nchunks, RL0_ROWS_CHUNK, 0, s>>>(a, nullptr, 0, 1);
     k_start<<<1, 32, 0, s>>>(a, 0, 1);
     cudaError_t e = cudaSuccess;
+    int rc = RL0_OK;
     for (int r = 0; r < nrounds && e == cudaSuccess; ++r) {
         e = mark(4 * r);
-        launch_column_score(a, indicator, learned, s);
+        if ((rc = launch_column_score(a, indicator, learned, s))) break;
         if (e == cudaSuccess) e = mark(4 * r + 1);
         if (e == cudaSuccess) e = mark(4 * r + 2);
         launch_rebuild(a, s);
@@ -629,7 +637,10 @@ int capture_decode_graph(rl0_expander *A, int nrounds, int indicator, int profil
     }
     if (e == cudaSuccess) e = mark(4 * nrounds);
     cudaError_t e2 = cudaStreamEndCapture(s, &g);
-    if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return rl0_cuda_err(e); }
+    if (rc || e != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return rc ? rc : rl0_cuda_err(e);
+    }
     if (e2 != cudaSuccess) return rl0_cuda_err(e2);
     e = cudaGraphInstantiate(&E->exec, g, 0);
     cudaGraphDestroy(g);
@@ -899,7 +910,7 @@ static int launch_analytic_continuation(rl0_expander *A, const KArgs &a, int64_t
     k_start<<<1, 32, 0, s>>>(a, 0, 0);
     k_list_count_from_support<<<1, 32, 0, s>>>(a);
     launch_bucket_support(a, s);
-    for (int r = 0; r < R2.nrounds; ++r) launch_round(a, R2.indicator, 0, s);
+    for (int r = 0; r < R2.nrounds; ++r) RC(launch_round(a, R2.indicator, 0, s));
     k_final_sum<<<1, 32, 0, s>>>(a);
     CK(cudaGetLastError());
     *launches = 5 + kernels_per_round(a, 0) * R2.nrounds + 1;
@@ -935,7 +946,7 @@ static int decode_adaptive(rl0_expander *A, const float *y_dev, int64_t k, const
     for (int r = 0; r < H->st.round && r < RL0_MAX_ROUNDS; ++r) H->kprior[r] = kprior;   // recorded rounds
     while (H->st.round < R.nrounds && !H->st.done) {
         const int r0 = H->st.round;
-        launch_round(a, R.indicator, 0, s);
+        RC(launch_round(a, R.indicator, 0, s));
         launches += kernels_per_round(a, 0);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(&H->st, w.st, sizeof(DecodeState), cudaMemcpyDeviceToHost, s));
@@ -1297,7 +1308,7 @@ extern "C" int rl0_round_step(const rl0_expander *Ac, const float *y_dev, int64_
     k_start<<<1, 32, 0, s>>>(a, round_index, 0);
     k_list_count_from_support<<<1, 32, 0, s>>>(a);
     launch_bucket_support(a, s);
-    launch_round(a, R.indicator, R.p.scorer == 1, s);
+    RC(launch_round(a, R.indicator, R.p.scorer == 1, s));
     k_extract_r<<<2 * a.nsm, 256, 0, s>>>(a, rp_dev, 0);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&H->st, w.st, sizeof(DecodeState), cudaMemcpyDeviceToHost, s));
@@ -1451,9 +1462,7 @@ extern "C" int rl0_decode_static(const rl0_expander *Ac, const float *y_dev, int
 
     k_rows_from<<<a.nchunks, RL0_ROWS_CHUNK, 0, s>>>(a, nullptr, 0, 1);
     k_start<<<1, 32, 0, s>>>(a, 0, 1);
-    for (int r = 0; r < R.nrounds; ++r) {
-        launch_round(a, R.indicator, R.p.scorer == 1, s);
-    }
+    for (int r = 0; r < R.nrounds; ++r) RC(launch_round(a, R.indicator, R.p.scorer == 1, s));
     k_final_sum<<<1, 32, 0, s>>>(a);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&H->st, base + L.st, sizeof(DecodeState), cudaMemcpyDeviceToHost, s));

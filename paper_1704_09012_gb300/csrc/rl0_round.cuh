@@ -537,10 +537,10 @@ __device__ void accept_step(const KArgs &a, unsigned upd, unsigned *shu)
 // (res_ok = 0 when the codes do not fit the device's shared memory or the
 // workspace has no code buffers); rl0_res_launch launches it (the learned
 // scorer's variant when learned is set) and returns false when a.res_ok is 0.
-// rl0_l2_launch launches the kernel that gathers from L2 (rl0_column_l2.cu).
 void rl0_res_setup(const rl0_expander *A, KArgs *a);
 int rl0_res_dmax(int d);                     // slots per survivor-list entry for degree d
 bool rl0_res_launch(const KArgs &a, int indicator, int learned, cudaStream_t s);
-// rl0_l2_setup sets its launch shape.
+// The kernel that gathers from L2 (rl0_column_l2.cu): rl0_l2_setup sets its launch
+// shape; rl0_l2_launch launches it, or returns RL0_ERR_CUDA when it has none.
 void rl0_l2_setup(KArgs *a);
-bool rl0_l2_launch(const KArgs &a, int indicator, int learned, cudaStream_t s);
+[[nodiscard]] int rl0_l2_launch(const KArgs &a, int indicator, int learned, cudaStream_t s);
