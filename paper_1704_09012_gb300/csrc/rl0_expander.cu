@@ -461,18 +461,21 @@ __global__ void __launch_bounds__(32 * RL0_SK_WARPS) k_sketch(int m, const int32
     __shared__ unsigned nzm[RL0_SK_WARPS][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
-    const int32_t b = rowptr[min(i, m)], e = rowptr[min(i + 1, m)];
-    const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)(e - b));
+    // places in a row are counted from its start (unsigned: a place past a row's end, up to the
+    // longest row's, added to the row's start could pass 2^31)
+    const int32_t b = (i < m) ? rowptr[i] : 0;
+    const unsigned len = (i < m) ? (unsigned)(rowptr[i + 1] - b) : 0u;
+    const unsigned longest = __reduce_max_sync(0xffffffffu, len);
     double acc = 0.0;
-    for (int c0 = 0; c0 < longest; c0 += 32 * RL0_SK_WARPS) {
-        const int c = c0 + 32 * wid;
+    for (unsigned c0 = 0; c0 < longest; c0 += 32 * RL0_SK_WARPS) {
+        const unsigned c = c0 + 32 * wid;
         unsigned mine = 0u;                         // lane q: the nonzero entries of row q
         if (c < longest) {
 #pragma unroll 16
             for (int q = 0; q < 32; ++q) {
-                const int32_t rb = __shfl_sync(0xffffffffu, b, q), re = __shfl_sync(0xffffffffu, e, q);
-                const int32_t p = rb + c + lane;
-                const float v = (p < re) ? __ldg(x + __ldg(colidx + p)) : 0.0f;
+                const int32_t rb = __shfl_sync(0xffffffffu, b, q);
+                const unsigned rl = __shfl_sync(0xffffffffu, len, q), p = c + lane;
+                const float v = (p < rl) ? __ldg(x + __ldg(colidx + rb + p)) : 0.0f;
                 const unsigned nz = __ballot_sync(0xffffffffu, v != 0.0f);
                 if (nz) sh[wid][q][lane] = v;
                 if (lane == q) mine = nz;
