@@ -75,11 +75,10 @@ __device__ __forceinline__ McHist mc_open(unsigned *sh, int nbins, int C)
     return McHist{sh, nbins, C, (int)(threadIdx.x & (C - 1))};
 }
 
-// Rows: bin |yhat_i|; event y0_i == 0; posterior p_breve_z(yhat_i).  Also writes
-// (yhat_i, y0_i) side by side for the pairs' gathers.
+// Rows: bin |yhat_i|; event y0_i == 0; posterior p_breve_z(yhat_i).
 __global__ void __launch_bounds__(RL0_MC_NT) k_mc_rows(int m, const float *__restrict__ y0,
-                                                       const float *__restrict__ yh, float2 *__restrict__ both,
-                                                       Series pz, int nbins, int C, float inv_w, unsigned long long *hz)
+                                                       const float *__restrict__ yh, Series pz, int nbins, int C,
+                                                       float inv_w, unsigned long long *hz)
 {
     extern __shared__ unsigned sh[];
     const McHist H = mc_open(sh, nbins, C);
@@ -89,7 +88,6 @@ __global__ void __launch_bounds__(RL0_MC_NT) k_mc_rows(int m, const float *__res
         const int i = i0 + threadIdx.x;
         if (i < m) {
             const float w = yh[i], z = y0[i];
-            both[i] = make_float2(w, z);
             const float a = fabsf(w) * inv_w;
             if (a < (float)nbins) mc_add(H, a, z == 0.0f, series_eval(pz, w));
         }
@@ -104,12 +102,17 @@ __global__ void __launch_bounds__(RL0_MC_NT) k_mc_rows(int m, const float *__res
 // Row pairs of every column (rows ascending, s < l): bin |yhat_s - yhat_l|;
 // event y0_s == y0_l; posterior p_breve_e(yhat_s - yhat_l).  One thread per
 // column, its d values in registers (slot-major row ids: coalesced).  n = 2^20,
-// d = 7 (22 M pairs), 64 bins: 434 us with three 64-bit atomics per pair on one
-// copy of the bins -> 153 us (series and conversions, by issue).
+// d = 7 (22 M pairs), 64 bins: the call took 444 us with three 64-bit atomics per
+// pair on one copy of the bins, now 206.  Two gathers per row: with (yhat, y0)
+// written side by side by the row kernel, one gather, it took 183, but the pairs
+// need memory of the call's own for that.  The expander's workspace is not it (a
+// decode, or another of these calls, may run on another stream), and a
+// stream-ordered allocation takes 200 us in every call that is waited for.
 template <int DMAX>
 __global__ void __launch_bounds__(RL0_MC_NT) k_mc_pairs(int n, int d, const int32_t *__restrict__ rows_sm,
-                                                        const float2 *__restrict__ both, Series pe, int nbins, int C,
-                                                        float inv_w, unsigned long long *he)
+                                                        const float *__restrict__ y0, const float *__restrict__ yh,
+                                                        Series pe, int nbins, int C, float inv_w,
+                                                        unsigned long long *he)
 {
     extern __shared__ unsigned sh[];
     const McHist H = mc_open(sh, nbins, C);
@@ -120,8 +123,13 @@ __global__ void __launch_bounds__(RL0_MC_NT) k_mc_pairs(int n, int d, const int3
         if (j < n) {
             float2 v[DMAX];
 #pragma unroll
-            for (int s = 0; s < DMAX; ++s)
-                v[s] = (s < d) ? __ldg(both + __ldg(rows_sm + (size_t)s * n + j)) : make_float2(0.0f, 0.0f);
+            for (int s = 0; s < DMAX; ++s) {
+                v[s] = make_float2(0.0f, 0.0f);
+                if (s < d) {
+                    const int i = __ldg(rows_sm + (size_t)s * n + j);
+                    v[s] = make_float2(__ldg(yh + i), __ldg(y0 + i));
+                }
+            }
 #pragma unroll
             for (int s = 0; s < DMAX; ++s) {
 #pragma unroll
@@ -167,15 +175,13 @@ extern "C" int rl0_posterior_mc(const rl0_expander *A, const float *y0_dev, cons
     const long long ctas = (long long)nsm * std::min(8, 2 * RL0_MC_SMEM / smem);
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if ((rc = rl0_cuda_err(cudaFuncSetAttribute(k_mc_rows, at, RL0_MC_SMEM)))) return rc;
-    // (yhat, y0) of every row side by side: the workspace is free between decodes
-    float2 *both = A->ws.rz[0];
     const int gr = (int)std::min<long long>(rl0_div_up(A->m, RL0_MC_NT), ctas);
     const int gp = (int)std::min<long long>(rl0_div_up(A->n, RL0_MC_NT), ctas);
-    k_mc_rows<<<gr, RL0_MC_NT, smem, s>>>((int)A->m, y0_dev, yhat_dev, both, pz, nbins, C, (float)(nbins / wz_max),
+    k_mc_rows<<<gr, RL0_MC_NT, smem, s>>>((int)A->m, y0_dev, yhat_dev, pz, nbins, C, (float)(nbins / wz_max),
                                           (unsigned long long *)hz_dev);
 #define RL0_MP(D) do {                                                                                              \
         if ((rc = rl0_cuda_err(cudaFuncSetAttribute(k_mc_pairs<D>, at, RL0_MC_SMEM)))) return rc;                   \
-        k_mc_pairs<D><<<gp, RL0_MC_NT, smem, s>>>((int)A->n, A->d, A->rows_sm, both, pe, nbins, C,                  \
+        k_mc_pairs<D><<<gp, RL0_MC_NT, smem, s>>>((int)A->n, A->d, A->rows_sm, y0_dev, yhat_dev, pe, nbins, C,                  \
                                                   (float)(nbins / we_max), (unsigned long long *)he_dev);           \
     } while (0)
     if (A->d <= 8) RL0_MP(8);
