@@ -84,9 +84,9 @@ __global__ void __launch_bounds__(RL0_MC_NT) k_mc_rows(int m, const float *__res
     const McHist H = mc_open(sh, nbins, C);
     const int every = mc_steps(C, 1);
     int steps = 0;
-    for (int i0 = blockIdx.x * RL0_MC_NT; i0 < m; i0 += gridDim.x * RL0_MC_NT) {
-        const int i = i0 + threadIdx.x;
-        if (i < m) {
+    for (unsigned i0 = blockIdx.x * RL0_MC_NT; i0 < (unsigned)m; i0 += gridDim.x * RL0_MC_NT) {   // (may pass 2^31)
+        const unsigned i = i0 + threadIdx.x;
+        if (i < (unsigned)m) {
             const float w = yh[i], z = y0[i];
             const float a = fabsf(w) * inv_w;
             if (a < (float)nbins) mc_add(H, a, z == 0.0f, series_eval(pz, w));
@@ -118,9 +118,9 @@ __global__ void __launch_bounds__(RL0_MC_NT) k_mc_pairs(int n, int d, const int3
     const McHist H = mc_open(sh, nbins, C);
     const int every = mc_steps(C, max(1, d * (d - 1) / 2));
     int steps = 0;
-    for (int j0 = blockIdx.x * RL0_MC_NT; j0 < n; j0 += gridDim.x * RL0_MC_NT) {
-        const int j = j0 + threadIdx.x;
-        if (j < n) {
+    for (unsigned j0 = blockIdx.x * RL0_MC_NT; j0 < (unsigned)n; j0 += gridDim.x * RL0_MC_NT) {
+        const unsigned j = j0 + threadIdx.x;
+        if (j < (unsigned)n) {
             float2 v[DMAX];
 #pragma unroll
             for (int s = 0; s < DMAX; ++s) {
