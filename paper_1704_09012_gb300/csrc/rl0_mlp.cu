@@ -71,6 +71,11 @@ __global__ void k_mlp_init(unsigned long long seed, float *w)
 // 4096-row minibatch took 35 us here, now 8.8 us.
 #define RL0_MLP_BLOCK 128
 #define RL0_MLP_WARPS (RL0_MLP_BLOCK / 16)
+// CTAs of a pass over more blocks than that: the GB300's 152 SMs (one CTA with the
+// gradient's shared memory fits each, four without).  Constants, not the device's
+// count: they set the order of the sums, which is the same on any device.
+#define RL0_MLP_GRAD_CTAS 152
+#define RL0_MLP_LOSS_CTAS 608
 #define RL0_MLP_FWD_FRAGS 12                                // W1: 4 n-tiles; W2: 2 k-steps x 4 n-tiles
 #define RL0_MLP_FRAGS 20                                    // and W2^T: 2 k-steps x 4 n-tiles
 #define RL0_MLP_FRAG_WORDS (RL0_MLP_FRAGS * 3 * 64)         // two words per lane, three parts
@@ -533,14 +538,6 @@ __global__ void __launch_bounds__(256) k_mlp_forward(const __nv_bfloat16 *wb, co
 // ---------------------------------------------------------------------------
 static const unsigned kRedGrid = (RL0_MLP_PARAMS + RL0_MLP_RED - 1) / RL0_MLP_RED;
 
-static int sm_count()
-{
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return nsm > 0 ? nsm : 1;
-}
-
 static int mlp_blocks(long long N) { return (int)((N + RL0_MLP_BLOCK - 1) / RL0_MLP_BLOCK); }
 
 // The limit on dynamic shared memory (an attribute of the kernels, set before use).
@@ -570,7 +567,7 @@ extern "C" int rl0_mlp_grad(const float *w_dev, const float *feat_dev, const flo
     cudaStream_t s = (cudaStream_t)cuda_stream;
     int rc = mlp_smem_limit();
     if (rc) return rc;
-    const int grid = std::min(mlp_blocks(N), sm_count());
+    const int grid = std::min(mlp_blocks(N), RL0_MLP_GRAD_CTAS);
     // one block: CTA partials, packed fragments, loss partials, the loss
     const size_t o_frag = (size_t)grid * RL0_MLP_PITCH * sizeof(float);
     const size_t o_lp = o_frag + RL0_MLP_FRAG_WORDS * sizeof(unsigned), o_ld = o_lp + (size_t)grid * sizeof(double);
@@ -603,7 +600,7 @@ extern "C" int rl0_mlp_train(float *w_dev, const float *feat_dev, const float *l
     if (rc) return rc;
     // a minibatch: one block per CTA; the final loss: resident CTAs (no gradient: the
     // weights' fragments are all the shared memory they use)
-    const int gmax = mlp_blocks(std::min<int64_t>(N, batch)), gall = std::min(mlp_blocks(N), 4 * sm_count());
+    const int gmax = mlp_blocks(std::min<int64_t>(N, batch)), gall = std::min(mlp_blocks(N), RL0_MLP_LOSS_CTAS);
     // one block: CTA partials, packed fragments, Adam's moments, loss partials, the loss
     const size_t o_frag = (size_t)gmax * RL0_MLP_PITCH * sizeof(float);
     const size_t o_m = o_frag + RL0_MLP_FRAG_WORDS * sizeof(unsigned), o_v = o_m + RL0_MLP_PITCH * sizeof(float);
