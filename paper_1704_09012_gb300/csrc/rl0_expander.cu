@@ -380,9 +380,11 @@ __global__ void __launch_bounds__(RL0_CSR_ROWS_NT) k_csr_rows(int m, CsrPlan P, 
     for (int p = t; p < E; p += RL0_CSR_ROWS_NT) colidx[g0 + p] = cols[p];
 }
 
-// The same with a global counter per row and an insertion sort per row: more
-// entries (n d above about 36 million) or rows (m above about a million) than the
-// buckets take.
+// The same with a global counter per row and an insertion sort per row, for what the
+// buckets do not take (rl0_expander_finish): buckets of more than 1024 rows (m above
+// a million, or fewer than about two entries per row), more entries per bucket than a
+// CTA's shared memory holds beside its counters (n d above 43 million at small m, 20
+// million at m = 10^6), or a row in its bucket and a column that do not share 32 bits.
 __global__ void k_row_count(int64_t nnz, const int32_t *rows_cm, int32_t *cnt1)
 {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
