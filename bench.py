@@ -142,7 +142,7 @@ class ClockSampler:
 # The sources that define the column kernel (its translation unit and the
 # headers it includes): the recorded DRAM traffic is reported only while these
 # are unchanged since the capture.
-COLUMN_KERNEL_SOURCES = ["rl0_column_res.cu", "rl0_resolve.cuh", "rl0_round.cuh", "rl0_device.cuh", "rl0_common.cuh"]
+COLUMN_KERNEL_SOURCES = ["rl0_column_res.cu", "rl0_resolve.cuh", "rl0_mma.cuh", "rl0_round.cuh", "rl0_device.cuh", "rl0_common.cuh"]
 
 
 def _code_only(src):

@@ -89,9 +89,8 @@ typedef struct {
     /* profile = 1 only: summed device time of each kernel group over the rounds the decode
      * ran (event nodes around the groups, so each interval includes the launch gap) */
     float   ms_score;          /* column scoring, with H_k in the kernel's last CTA          */
-    float   ms_hk;             /* from the scoring kernel's end to the scatter's start       */
-    float   ms_rebuild;        /* scatter + residual rebuild, with accept/undo in the        */
-                               /* rebuild's last CTA                                         */
+    float   ms_hk;             /* from the scoring kernel's end to the rebuild's start       */
+    float   ms_rebuild;        /* residual rebuild, with accept/undo in its last CTA         */
     float   ms_accept;         /* from the rebuild's end to the next round's start           */
     int     launches;          /* kernels launched by the decode (any mode)                  */
     int     analytic_rounds;   /* scorer = 1: rounds of the analytic continuation (0 if the  */

@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
     // the first tile's row ids while the previous kernel finishes (A never changes)
     int nxt[DMAX];
 #pragma unroll
-    for (int s = 0; s < DMAX; ++s) nxt[s] = (s < d && lo + tid < hi) ? __ldg(a.rows_sm + (size_t)s * n + lo + tid) : 0;
+    for (int s = 0; s < DMAX; ++s) nxt[s] = (lo + tid < hi) ? __ldg(a.rows_sm + (size_t)s * n + lo + tid) : 0;
     pdl_wait();                                    // the previous rebuild's r, x and state
     const int done = st->done, cur = st->cur, round = st->round, look = st->look;
     const unsigned nnz0 = st->nnz;
@@ -118,20 +118,20 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
 #pragma unroll
             for (int s = 0; s < DMAX; ++s) {
                 v[s] = make_float2(0.0f, 0.0f);
-                if (s < d && active) v[s] = __ldca(rz + rid[s]);
+                if (active) v[s] = __ldca(rz + rid[s]);
             }
             {
                 const int jn = j + NT;
 #pragma unroll
                 for (int s = 0; s < DMAX; ++s)
-                    if (s < d && jn < hi) nxt[s] = __ldg(a.rows_sm + (size_t)s * n + jn);
+                    if (jn < hi) nxt[s] = __ldg(a.rows_sm + (size_t)s * n + jn);
             }
             float r[DMAX];
             float nz = 0.0f;
 #pragma unroll
             for (int s = 0; s < DMAX; ++s) {
                 r[s] = v[s].x;
-                if (s < d) nz += IND ? (fabsf(v[s].x) <= th.tz ? 1.0f : 0.0f) : v[s].y;
+                nz += IND ? (fabsf(v[s].x) <= th.tz ? 1.0f : 0.0f) : v[s].y;
             }
             const unsigned cm = active ? anchor_candidates<DMAX, IND>(r, d, ta_look, reach, b1, c1, nz, need) : 0u;
             const unsigned m = __ballot_sync(0xffffffffu, cm != 0u);
@@ -173,12 +173,12 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
                 old = __ldca(xg + j);
                 const int *ids = a.rows_cm + (size_t)j * d;
 #pragma unroll
-                for (int s = 0; s < DMAX; ++s) v[s] = (s < d) ? __ldca(rz + __ldg(ids + s)) : make_float2(0.0f, 0.0f);
+                for (int s = 0; s < DMAX; ++s) v[s] = __ldca(rz + __ldg(ids + s));
             }
             auto rows = [&](int *rid) {
                 const int *ids = a.rows_cm + (size_t)j * d;
 #pragma unroll
-                for (int s = 0; s < DMAX; ++s) rid[s] = (s < d) ? __ldg(ids + s) : 0;
+                for (int s = 0; s < DMAX; ++s) rid[s] = __ldg(ids + s);
             };
             resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, ta_look, round, d, rule, alpha, passed, M.R, S, act, j, cm,
                                                   old, v, rows);

@@ -29,8 +29,8 @@
 //   H_k      the launch's last CTA (a 64-bit acquire-release ticket that also
 //            sums the CTAs' changes of the nonzero count) applies H_k
 //            when |supp x'| > k, its scratch in the bytes that held the codes.
-// The resolve runs the arithmetic of k_column_score in the same order, so
-// both kernels give the same x'.
+// The resolve is the one of rl0_column_l2.cu (rl0_resolve.cuh), so both kernels
+// give the same x'.
 #include <algorithm>
 
 #include "rl0_common.cuh"

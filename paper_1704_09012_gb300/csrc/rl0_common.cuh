@@ -79,18 +79,18 @@ struct DecodeState {
     int nnz_delta;            // change of the nonzero count made by this round's updates
     unsigned zeroed;          // updates that made an entry exactly zero this round
     unsigned iters;           // accept invocations (bounds the graph's while loop)
-    unsigned col_done;        // CTAs of the column kernel finished (last one applies H_k)
+    unsigned col_done;        // CTAs of the tile column kernel finished (last one applies H_k)
     unsigned rb_done;         // CTAs of the rebuild finished (last one accepts or undoes)
     unsigned big_hat;         // Alg. 1 mode: rows of r_hat with |r_i| > conv_tol
     unsigned big_cand;        // Alg. 1 mode: the same count for the candidate r
-    int skipped;              // rounds recorded without running their kernels (the t = 1 round)
+    int skipped;              // rounds recorded without running their kernels (rl0_round.cuh)
     int rounds_run;
     int accepted_rounds;
     int hk_rounds;
     int fallback_rounds;
     int look;                 // the next round's column pass looks ahead (see rl0_round.cuh)
     int next_event;           // looking ahead: the first later round in which a column would pass
-    unsigned long long tick;  // resident-code column kernel: CTAs done (bits 48..63) and their
+    unsigned long long tick;  // resident CTAs' column kernels: CTAs done (bits 48..63) and their
                               // changes of the nonzero count, each biased by 2^31 (bits 0..47)
     double l1_hat;
     double l1_new;

@@ -3,16 +3,15 @@
 // coefficients (host, FP64), the round kernels, and the captured CUDA graph
 // that replays the loop.
 //
-// One round, as two or three kernels on one stream:
+// One round, as two kernels on one stream:
 //   column score  every column j bounds, then scores, its anchors (Table
 //                 "scores", Eqs. (ne_nz_1), (ne_nz_2)), applies the last
 //                 passing update to x in place and logs it for undo
-//                 (k_column_score_res in rl0_column_res.cu: residual codes in
-//                 shared memory; k_column_score below: L2 gathers).  The
-//                 launch's last CTA applies H_k (radix select on the 63-bit
-//                 key (|x_j| bits, ~j): ties go to the smaller j);
-//   scatter       the support's (row, column) pairs into per-row buckets
-//                 (the resident-code column kernel does this itself);
+//                 (rl0_column_res.cu: residual codes in shared memory;
+//                 rl0_column_l2.cu: L2 gathers), and puts the columns that
+//                 became nonzero into per-row buckets.  The launch's last
+//                 CTA applies H_k (radix select on the 63-bit key
+//                 (|x_j| bits, ~j): ties go to the smaller j);
 //   rebuild       r_i = y_i - sum of x_j over row i in ascending j, FP32 (and
 //                 the same sum in FP32 pairs, about 48 bits, for the final
 //                 residual check), with p_z(r_i), the residual code, and l1
@@ -865,8 +864,8 @@ static int get_graph(rl0_expander *A, int nrounds, int indicator, int prof, int 
 }
 
 // The settings in H (ctx, pzlb, nrounds thresholds) to the device, with fresh, also
-// a zeroed decode state: one copy, where four (three and a memset) took about 2 us
-// each before the first kernel.
+// a zeroed decode state: one operation queued before the first kernel instead of
+// four (three copies and a memset).
 static cudaError_t upload_stage(const rl0_expander *A, int nrounds, bool fresh, cudaStream_t s)
 {
     HostStage *H = (HostStage *)A->host_pinned;
