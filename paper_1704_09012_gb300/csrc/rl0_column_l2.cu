@@ -15,12 +15,12 @@
 //            survives.  Other CTAs of the SM stream meanwhile.
 //   H_k      in the launch's last CTA, as in the resident-code kernel.
 // A queue scored by CTA-wide passes (one candidate slot per column and pass, two
-// barriers each) left the warps waiting for one another: 11 of 25 warp-cycles
-// per issue at n = 2^22, m = 419 430, d = 7, 19 of 27 with the learned scorer.
-// Full batches instead: a whole decode there (39 rounds) 8.62 -> 6.62 ms, a
-// learned one (78 rounds) 42.5 -> 33.7 ms, and at n = 2^24, m = 167 772 a round
-// 0.71 -> 0.54 ms.  What is left is the gathers: an SM asks L2 for about one
-// 32-byte sector per cycle, 0.1 ms for the 29 M of a round at n = 2^22.
+// barriers each) left the warps waiting for one another: barriers were 8.7 of 25.7
+// warp-cycles per issue at n = 2^22, m = 419 430, d = 7, 17 with the learned
+// scorer.  Full batches instead: a round there 218 -> 150 us (learned 790 -> 199,
+// with the packed network), a whole decode of 39 rounds 8.62 -> 6.59 ms, and at
+// n = 2^24, m = 167 772 a round 0.71 -> 0.54 ms.  What is left is the gathers: an
+// SM asks L2 for 0.8 32-byte sectors per cycle, 34 M in a round at n = 2^22.
 #include <algorithm>
 #include <type_traits>
 

@@ -103,7 +103,9 @@ __global__ void __launch_bounds__(RL0_MC_NT) k_mc_rows(int m, const float *__res
 // event y0_s == y0_l; posterior p_breve_e(yhat_s - yhat_l).  One thread per
 // column, its d values in registers (slot-major row ids: coalesced).  n = 2^20,
 // d = 7 (22 M pairs), 64 bins: the call took 444 us with three 64-bit atomics per
-// pair on one copy of the bins, now 206.  Two gathers per row: with (yhat, y0)
+// pair on one copy of the bins, now 206, 187 of them here (issue: half the slots are
+// busy, the warps wait for instructions of the unrolled pairs and for the queue of
+// shared-memory operations).  Two gathers per row: with (yhat, y0)
 // written side by side by the row kernel, one gather, it took 183, but the pairs
 // need memory of the call's own for that.  The expander's workspace is not it (a
 // decode, or another of these calls, may run on another stream), and a

@@ -68,7 +68,7 @@ __global__ void k_mlp_init(unsigned long long seed, float *w)
 // What bounds it is latency: one block's chain of products, with one block per
 // SM and 32 blocks in a minibatch of 4096.  Splitting operands inside the
 // products' loops (the weights by every warp, X and D by every output tile), a
-// 4096-row minibatch took 35 us here, now 8.8 us.
+// 4096-row minibatch took 34-39 us here, now 8.9 us.
 #define RL0_MLP_BLOCK 128
 #define RL0_MLP_WARPS (RL0_MLP_BLOCK / 16)
 // CTAs of a pass over more blocks than that: the GB300's 152 SMs (one CTA with the
@@ -485,8 +485,8 @@ __global__ void __launch_bounds__(RL0_MLP_RED) k_mlp_grad_reduce(const float *pa
 // partials add up to; the new weights go into the packed fragments as well.
 // One thread per parameter, its partials 16 loads at a time; the launches overlap
 // (features and moments load while the previous kernel finishes).  A 4096-row
-// step, both kernels alone (ncu): 35 + 5.4 -> 8.8 + 4.6 us; two epochs over
-// 400 003 rows with the final loss 8.66 -> 2.20 ms.
+// step, both kernels alone (ncu): 37 + 4.8 -> 8.9 + 4.3 us; two epochs over
+// 400 003 rows with the final loss 8.33 -> 2.19 ms.
 __global__ void __launch_bounds__(RL0_MLP_RED) k_mlp_reduce_adam(const float *part, int nparts, float *w, float *m,
                                                                  float *v, unsigned short *frag, int step, float lr,
                                                                  float b1, float b2, float eps)

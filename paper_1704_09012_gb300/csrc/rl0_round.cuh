@@ -53,10 +53,17 @@ struct KArgs {
 // little: a row of small |r| has p_z near 1, and n_z then rules its column out).
 // Sweeps that do not reach the stop level end this way: n = 2^24, delta = 0.01
 // updates in its first few rounds of 99 and scored all columns again in every
-// other.  Mean over instances that converge and instances that stall: n = 2^24
-// decode 24.3 -> 7.5 ms, n = 2^22 (rho = 0.15) 6.62 -> 4.44 ms, n = 2^20
-// 0.41 -> 0.26 ms, n = 4096 0.218 -> 0.141 ms, adaptive_k at n = 100003
-// 1.77 -> 0.97 ms.
+// other.  Without and with looking ahead, the rest the same, per call:
+//   stalls (d = 7)     n = 4096, k = 100 (7 of 39 rounds run)  398 -> 174 us
+//                      n = 4096, k = 250 (3 of 39)             431 -> 98 us
+//                      n = 2^20, k = 20971 (7 of 39)           849 -> 261 us
+//                      n = 2^22, m = 419430, 30 dB             6.59 -> 4.45 ms
+//                      n = 2^24, m = 167772                    53.6 -> 14.7 ms
+//                      adaptive_k, n = 100003, d = 10          1.78 -> 0.94 ms
+//   256 mixed instances, batched                               5.76 -> 5.01 ms
+// A decode that converges while it updates gains nothing (n = 2^20, k = 10485,
+// 40 dB, 7 of 7 rounds: 263 and 262 us), nor does one that updates in every
+// round (n = 2^22, 40 dB, 39 of 39: 10.6 ms).
 // ---------------------------------------------------------------------------
 #define RL0_LOOK_SHARE 256          // look ahead after a round of at most k / 256 updates
 

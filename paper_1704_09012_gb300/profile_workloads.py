@@ -21,6 +21,16 @@ range of its own name, so that a tool such as Nsight Compute can select it
       rl0_mlp_train); `reps` repetitions (default 2), each in a range "learned".  At
       n = 2^20 the round runs on the resident-code kernel, at n = 2^22 (whose codes do not
       fit in shared memory) on the L2-gather kernel.
+  python -m paper_1704_09012_gb300.profile_workloads gather [log2n] [reps]
+      one round with the analytic rule on the L2-gather kernel: the learned workload's
+      instance and state (default n = 2^22), in a range "gather";
+  python -m paper_1704_09012_gb300.profile_workloads posterior
+      one rl0_posterior_mc call at n = 2^20, m = 0.3 n, rho = 0.1, d = 7, sigma_n = 0.01,
+      64 bins, in a range "posterior";
+  python -m paper_1704_09012_gb300.profile_workloads train
+      rl0_mlp_train on 16384 rows, one pass of 4096-row minibatches, in a range "train";
+  python -m paper_1704_09012_gb300.profile_workloads build
+      rl0_make_expander at n = 2^22, m = 41943, d = 7, in a range "build".
 
 Every step of the decode runs in the CUDA library; torch only holds device memory and
 subtracts A x_hat from y_hat to form the injected residual."""
@@ -65,6 +75,15 @@ def learned_workload(log2n=20, reps=2):
         Y.append(lab)
         A.free()
     wb, _, _ = learned.train_scorer(torch.cat(F), torch.cat(Y), epochs=4)
+    _low_snr_round("learned", log2n, reps, scorer=1, mlp=wb)
+
+
+def gather_workload(log2n=22, reps=2):
+    _low_snr_round("gather", log2n, reps)
+
+
+def _low_snr_round(name, log2n, reps, **params):
+    d = 7
     n = 1 << log2n
     m = n // 10
     k = int(0.15 * m)
@@ -75,10 +94,40 @@ def learned_workload(log2n=20, reps=2):
     xh, _ = rl0.decode(A, y, k, sigma_n=sn, max_rounds=3)
     rh = y - rl0.sketch(A, xh, sigma_n=0.0)
     for _ in range(reps):
-        torch.cuda.nvtx.range_push("learned")
-        rl0.round_step(A, y, k, 3, xh, rh, want_passed=False, sigma_n=sn, scorer=1, mlp=wb)
+        torch.cuda.nvtx.range_push(name)
+        rl0.round_step(A, y, k, 3, xh, rh, want_passed=False, sigma_n=sn, **params)
         torch.cuda.nvtx.range_pop()
     torch.cuda.synchronize()
+
+
+def posterior_workload():
+    n, d, sn = 1 << 20, 7, 0.01
+    m = int(0.3 * n)
+    k = int(0.1 * m)
+    A = rl0.Expander.random(n, m, d, seed=300)
+    x, _ = gm.draw_signal(n, k, 1.0, 300)
+    xt = torch.from_numpy(x).cuda()
+    y0, y = rl0.sketch(A, xt), rl0.sketch(A, xt, sigma_n=sn, noise_seed=400)
+    torch.cuda.nvtx.range_push("posterior")
+    rl0.posterior_mc(A, y0, y, k, sn)
+    torch.cuda.nvtx.range_pop()
+    torch.cuda.synchronize()
+
+
+def train_workload():
+    g = torch.Generator("cuda").manual_seed(1)
+    F = torch.randn(16384, 16, generator=g, device="cuda")
+    y = (torch.rand(16384, generator=g, device="cuda") < 0.3).float()
+    w = rl0.mlp_init(seed=1)
+    torch.cuda.nvtx.range_push("train")
+    rl0.mlp_train(w, F, y, epochs=1, batch=4096)
+    torch.cuda.nvtx.range_pop()
+
+
+def build_workload():
+    torch.cuda.nvtx.range_push("build")
+    rl0.Expander.random(1 << 22, 41943, 7, seed=1)
+    torch.cuda.nvtx.range_pop()
 
 
 def batched_workload(count=256):
@@ -100,17 +149,16 @@ def batched_workload(count=256):
     torch.cuda.synchronize()
 
 
+WORKLOADS = {"round": round_workload, "batched": batched_workload, "learned": learned_workload, "gather": gather_workload,
+             "posterior": posterior_workload, "train": train_workload, "build": build_workload}
+
+
 def main(argv):
-    if not argv or argv[0] not in ("round", "batched", "learned"):
+    if not argv or argv[0] not in WORKLOADS:
         print(__doc__)
         return 2
     torch.cuda.set_device(0)
-    if argv[0] == "round":
-        round_workload(int(argv[1]) if len(argv) > 1 else 3)
-    elif argv[0] == "learned":
-        learned_workload(int(argv[1]) if len(argv) > 1 else 20, int(argv[2]) if len(argv) > 2 else 2)
-    else:
-        batched_workload(int(argv[1]) if len(argv) > 1 else 256)
+    WORKLOADS[argv[0]](*[int(v) for v in argv[1:]])
     print("%s workload done" % argv[0])
     return 0
 
