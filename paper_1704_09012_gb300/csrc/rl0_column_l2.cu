@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(L2NT<DMAX>::value, L2Occ<LEARNED>::value) k_co
                 for (int s = 0; s < DMAX; ++s) rid[s] = __ldg(ids + s);
             };
             resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, ta_look, round, d, rule, alpha, passed, M.R, S, act, j, cm,
-                                                  old, v, rows);
+                                                  old, v, rows, LEARNED ? (const MlpPacked *)&M.R.mlp : nullptr);
             head += min((unsigned)NT, cnt - head);
         }
     }

@@ -138,6 +138,19 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
             nxt[s] = (s < d && j < hi) ? __ldg(a.rows_sm + (size_t)s * n + j) : 0;
         }
     }
+    // the learned scorer's network likewise (no kernel of a decode writes it or its address).
+    // Packed where the resolve begins, it held up every round: learned decodes at n = 4096,
+    // m = 1024 475 -> 448 us, n = 15306, m = 2051 477 -> 446, n = 60000, m = 2400, d = 8
+    // 1211 -> 1159 (not packed at all 445, 442 and 1331; means over 12 expanders, whose
+    // places in memory make 5% of difference).
+    MlpSlice slice;
+    MlpPacked *early = nullptr;
+    if constexpr (LEARNED && NT >= 384) {
+        if (a.res_mlp_off) {
+            early = (MlpPacked *)(dsm + a.res_mlp_off);
+            mlp_fetch(slice, (const __nv_bfloat16 *)__ldcg((const unsigned long long *)&ctx->mlp), tid);
+        }
+    }
     pdl_wait();                                    // the previous rebuild's r, codes, x and state
     // done, cur and round in one L2 trip (the code copy waits on cur)
     const int done = st->done, cur = st->cur, round = st->round, look = st->look;
@@ -181,6 +194,9 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     const unsigned polls = ctx->wait_test ? ctx->wait_polls : RL0_RES_WAIT_LIMIT;
     __syncthreads();                               // the barrier is initialised
     const bool arrived = mbar_try_wait_bounded(bar, 0u, polls);
+    if constexpr (LEARNED && NT >= 384) {
+        if (early) mlp_store(*early, slice, tid);  // read after the barriers below
+    }
     if (__syncthreads_or(!arrived || __ldcg(&st->status) == (int)RL0_ERR_CUDA)) {
         // a copy did not complete in time: record it, wait for the copies in
         // flight once more (with the built-in limit) before this CTA's shared
@@ -203,8 +219,8 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     const int lane = tid & 31;
     // this CTA's survivors: the first qcap in shared memory, the others in its
     // slice of the global list, entries (j, candidate mask, its d row ids)
-    ResEntry<DMAX> *sq = (ResEntry<DMAX> *)(dsm + a.res_q_off);
-    const int qcap = a.res_qcap;
+    ResEntry<DMAX> *sq = (ResEntry<DMAX> *)(dsm + a.res_q_off[LEARNED]);
+    const int qcap = a.res_qcap[LEARNED];
     int *seg = a.res_list + (size_t)lo * (size_t)(DMAX + 2);
     const float *xg = ctx->x;
     // list column j (candidate mask cm, row ids rid) at position pos
@@ -333,9 +349,13 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
     __syncthreads();                               // the stream is done: the codes' bytes become scratch
     const int count = min(S.count, hi - lo);
     ResScratch<DMAX, NT, LEARNED> &R = *(ResScratch<DMAX, NT, LEARNED> *)dsm;
+    const MlpPacked *net = early;
     if constexpr (LEARNED) {                       // first read after the batch's barriers
         if (tid == 0) R.nf = 0;
-        if (count > 0) mlp_pack(R.mlp, (const __nv_bfloat16 *)ctx->mlp, tid, NT);
+        if (!early) {
+            net = &R.mlp;
+            if (count > 0) mlp_pack(R.mlp, (const __nv_bfloat16 *)ctx->mlp, tid, NT);
+        }
     }
     const float alpha = ctx->alpha;
     for (int b0 = 0; b0 < count; b0 += NT) {
@@ -374,7 +394,7 @@ __device__ __forceinline__ bool column_phase(const KArgs &a, unsigned char *dsm)
             }
         };
         resolve_batch<DMAX, IND, NT, LEARNED>(a, ctx, th, ta_look, round, d, rule, alpha, passed, R, S, act, j, cm, old, v,
-                                              rows);
+                                              rows, net);
     }
     if (!IND && !LEARNED && tid == 0 && S.next_event != 0x7fffffff) atomicMin(&st->next_event, S.next_event);
     return true;
@@ -454,18 +474,23 @@ void rl0_res_setup(const rl0_expander *A, KArgs *a)
     const unsigned region = res_region_bytes(A->m, nt, res_scratch_bytes(A->d));
     a->res_pz_off = region;
     a->res_s_off = region + 4u * RL0_PZ_BINS;
-    a->res_q_off = (a->res_s_off + (unsigned)sizeof(ColState) + 15u) & ~15u;
+    const unsigned q0 = (a->res_s_off + (unsigned)sizeof(ColState) + 15u) & ~15u;
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, A->device) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
-    if (a->res_q_off > (unsigned)optin) return;
+    if (q0 > (unsigned)optin) return;
     // the shared memory left over stages survivors (one CTA per SM: nothing
-    // else competes for it); the others go to the global list
-    const unsigned eb = res_entry_bytes(res_variant(A->d));
-    a->res_qcap = (int)std::min<unsigned>(((unsigned)optin - a->res_q_off) / eb, 4096u);
-    a->res_smem = a->res_q_off + (unsigned)a->res_qcap * eb;
+    // else competes for it); the others go to the global list.  The learned
+    // scorer's network comes before them where it fits.
+    const unsigned eb = res_entry_bytes(res_variant(A->d)), mb = ((unsigned)sizeof(MlpPacked) + 15u) & ~15u;
+    a->res_mlp_off = (q0 + mb <= (unsigned)optin) ? q0 : 0u;
+    for (int l = 0; l < 2; ++l) {
+        a->res_q_off[l] = q0 + (l && a->res_mlp_off ? mb : 0u);
+        a->res_qcap[l] = (int)std::min<unsigned>(((unsigned)optin - a->res_q_off[l]) / eb, 4096u);
+        a->res_smem[l] = a->res_q_off[l] + (unsigned)a->res_qcap[l] * eb;
+    }
     bool ok = false;
     switch (res_variant(A->d)) {
     case 6: ok = res_attr<6, true>(optin); break;
@@ -483,16 +508,17 @@ void rl0_res_setup(const rl0_expander *A, KArgs *a)
 bool rl0_res_launch(const KArgs &a, int indicator, int learned, cudaStream_t s)
 {
     if (!a.res_ok || (learned && a.d > 16)) return false;
-#define RL0_CR(D, E) do {                                                                                        \
-        constexpr int NT_ = ResNT<D, E>::value;                                                                   \
-        if (learned) {                                                                                            \
-            if (indicator) launch_pdl(k_column_score_res<D, true, E, NT_, true>, a.res_grid, NT_, a.res_smem, s, a); \
-            else launch_pdl(k_column_score_res<D, false, E, NT_, true>, a.res_grid, NT_, a.res_smem, s, a);      \
-        } else if (indicator) {                                                                                   \
-            launch_pdl(k_column_score_res<D, true, E, NT_, false>, a.res_grid, NT_, a.res_smem, s, a);            \
-        } else {                                                                                                  \
-            launch_pdl(k_column_score_res<D, false, E, NT_, false>, a.res_grid, NT_, a.res_smem, s, a);           \
-        }                                                                                                         \
+#define RL0_CR(D, E) do {                                                                                          \
+        constexpr int NT_ = ResNT<D, E>::value;                                                                     \
+        const unsigned sm = a.res_smem[learned ? 1 : 0];                                                            \
+        if (learned) {                                                                                              \
+            if (indicator) launch_pdl(k_column_score_res<D, true, E, NT_, true>, a.res_grid, NT_, sm, s, a);        \
+            else launch_pdl(k_column_score_res<D, false, E, NT_, true>, a.res_grid, NT_, sm, s, a);                 \
+        } else if (indicator) {                                                                                     \
+            launch_pdl(k_column_score_res<D, true, E, NT_, false>, a.res_grid, NT_, sm, s, a);                      \
+        } else {                                                                                                    \
+            launch_pdl(k_column_score_res<D, false, E, NT_, false>, a.res_grid, NT_, sm, s, a);                     \
+        }                                                                                                           \
     } while (0)
     switch (res_variant(a.d)) {
     case 6: RL0_CR(6, true); break;

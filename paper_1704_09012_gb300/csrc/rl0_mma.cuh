@@ -106,8 +106,9 @@ struct MlpGlobal {
 // 8-byte word, the vectors in FP32.  From global memory a tile of 16 rows takes
 // 48 two-byte loads of four cache lines each for the fragments and 25 more.
 // Packed, and with the features' seven smallest deviations kept in registers
-// (rl0_device.cuh): learned decodes at n = 15306, d = 7 447 -> 425 us, at n = 201716,
-// d = 9 1137 -> 1039 us, at n = 2^22, d = 7 (gathers from L2) 33.5 -> 32.6 ms.
+// (rl0_device.cuh): learned decodes at n = 60000, d = 8 1331 -> 1159 us, at n = 201716,
+// d = 9 1047 -> 906 us, at n = 2^22, d = 7 (gathers from L2) 33.5 -> 32.6 ms; with few
+// candidates (n = 15306) no change, 442 and 446 us.
 struct MlpPacked {
     uint2 w[12][32];
     float2 b1[RL0_HID / 2], b2[RL0_HID / 2], w3[RL0_HID / 2];
@@ -141,6 +142,32 @@ __device__ __forceinline__ void mlp_pack(MlpPacked &P, const __nv_bfloat16 *wb, 
         P.w3[tid] = G.pair(RL0_OFF_W3, 2 * tid);
     }
     if (tid == 0) P.b3v = G.b3();
+}
+
+// The same in two halves for a CTA of at least 384 threads: the loads (a thread's
+// fragment and vector words, in registers), and the stores into P.
+struct MlpSlice {
+    unsigned b[2];
+    float2 v;
+    float b3v;
+};
+
+__device__ __forceinline__ void mlp_fetch(MlpSlice &L, const __nv_bfloat16 *wb, int tid)
+{
+    const MlpGlobal G{wb};
+    const int lane = tid & 31, i = tid >> 5;
+    if (i < 12) G.frag(i, L.b);
+    // warps 0-2: b1, b2, w3
+    if (i < 3 && lane < RL0_HID / 2) L.v = G.pair(i == 0 ? RL0_OFF_B1 : i == 1 ? RL0_OFF_B2 : RL0_OFF_W3, 2 * lane);
+    if (tid == 0) L.b3v = G.b3();
+}
+
+__device__ __forceinline__ void mlp_store(MlpPacked &P, const MlpSlice &L, int tid)
+{
+    const int lane = tid & 31, i = tid >> 5;
+    if (i < 12) P.w[i][lane] = make_uint2(L.b[0], L.b[1]);
+    if (i < 3 && lane < RL0_HID / 2) (i == 0 ? P.b1 : i == 1 ? P.b2 : P.w3)[lane] = L.v;
+    if (tid == 0) P.b3v = L.b3v;
 }
 
 // Logits of 16 rows with the parameters W (MlpGlobal or MlpPacked: the same

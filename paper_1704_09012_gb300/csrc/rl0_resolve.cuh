@@ -81,13 +81,13 @@ __device__ __forceinline__ unsigned cta_exclusive_scan(unsigned v, unsigned *wsu
 // slots cm, x_j and the (r, p_z) of its rows in v; rows(rid) gives the column's
 // row ids.  ta_look: the anchors to test (th.ta, or the sweep's last t_a when
 // the pass looks ahead; those below th.ta only report the round that makes
-// them anchors).  Every thread of the CTA calls it; the scratch is free again when
-// it returns.  The arithmetic is eval_anchor's, in its order.
+// them anchors).  net: the learned scorer's network, in shared memory.  Every thread
+// of the CTA calls it; the scratch is free again when it returns.  The arithmetic is eval_anchor's, in its order.
 template <int DMAX, bool IND, int NT, bool LEARNED, class Rows>
 __device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *ctx, const RoundThr &th, float ta_look,
                                               int round, int d, int rule, float alpha, int32_t *passed, ResScratch<DMAX, NT, LEARNED> &R,
                                               ColState &S, bool act, int j, unsigned cm, float old, const float2 *v,
-                                              Rows rows)
+                                              Rows rows, const MlpPacked *net = nullptr)
 {
     constexpr bool LOOK = !IND && !LEARNED;
     const int tid = threadIdx.x;
@@ -179,7 +179,7 @@ __device__ __forceinline__ void resolve_batch(const KArgs &a, const DecodeCtx *c
             for (unsigned t0 = (unsigned)(tid >> 5) * 16u; t0 < nf; t0 += (NT / 32) * 16u) {
                 auto f = [&](int r, int i) { return (t0 + r < nf && i < RL0_NFEAT - 2) ? R.feat[i][t0 + r] : 0.0f; };
                 float lo, hi;
-                warp_mlp_logits16(f, R.mlp, &lo, &hi);
+                warp_mlp_logits16(f, *net, &lo, &hi);
                 if ((tid & 3) == 0) {
                     const unsigned gr = (unsigned)((tid & 31) >> 2);
                     if (t0 + gr < nf && !(lo >= ctx->logit_thr)) R.it_ok[k0 + R.fidx[t0 + gr]] = 0;

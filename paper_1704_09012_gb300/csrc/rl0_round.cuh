@@ -20,10 +20,12 @@ struct KArgs {
     const float *pzlb;                 // p_z lower bound per code bin
     int res_ok;                        // the column kernel holds every row's code in shared memory
     int res_grid;                      // its CTAs (one per SM)
-    unsigned res_pz_off, res_s_off, res_q_off, res_smem;   // its dynamic shared-memory layout
+    unsigned res_pz_off, res_s_off;    // its dynamic shared-memory layout ...
+    unsigned res_mlp_off;              // (learned) the network's place in it (0: none left, it goes into the scratch)
+    unsigned res_q_off[2], res_smem[2];   // ... the staged survivors and the total: analytic, learned
     int l2_grid[2];                    // CTAs of the L2-gather column kernel: analytic, learned (0: no variant)
     unsigned l2_smem[2];               // its dynamic shared memory
-    int res_qcap;                      // survivors per CTA staged in shared memory (FP32 residuals and x_j)
+    int res_qcap[2];                   // survivors per CTA staged in shared memory (FP32 residuals and x_j)
     int *res_list;                     // its other survivors: n entries of (j, candidate mask, DMAX row ids);
                                        // CTA b uses its column range
     int *list;
