@@ -94,7 +94,7 @@ struct DecodeState {
                               // changes of the nonzero count, each biased by 2^31 (bits 0..47)
     double l1_hat;
     double l1_new;
-    double final_l1;          // ||y_hat - A x_hat||_1 in FP64 (epilogue)
+    double final_l1;          // ||y_hat - A x_hat||_1 in FP64 (epilogue); last: the accept step reads what is before it
 };
 
 // Per-call data the round kernels read from device memory.  The graph that

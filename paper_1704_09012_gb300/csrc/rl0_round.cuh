@@ -369,11 +369,12 @@ __device__ __forceinline__ bool rebuild_row(const KArgs &a, const DecodeCtx *ctx
 template <int NT>
 __device__ void accept_step(const KArgs &a, unsigned upd, unsigned *shu)
 {
-    // The state is read once into shared memory (one word per thread,
+    // The state is read once into shared memory (warp 0, one word per lane,
     // through L2: other CTAs of this launch wrote to it), decided on there,
     // and written back once, so thread 0's decisions wait on no global loads.
-    constexpr int SW = sizeof(DecodeState) / 4;
-    static_assert(sizeof(DecodeState) % 4 == 0 && SW <= NT, "one word per thread");
+    // final_l1, written here and read by nobody, lies past that line.
+    constexpr int SW = offsetof(DecodeState, final_l1) / 4;
+    static_assert(offsetof(DecodeState, final_l1) % 4 == 0 && SW <= 32, "one word per lane of warp 0");
     __shared__ DecodeState S;
     __shared__ double s_l1;
     __shared__ int s_acc;
@@ -534,7 +535,7 @@ __device__ void accept_step(const KArgs &a, unsigned upd, unsigned *shu)
         // the decode ends here: ||y_hat - A x_hat||_1 from r_hat's chunk
         // partials, in k_final_sum's order
         const double fv = cta_sum_parts_l2<NT>(a.final_part + (size_t)S.cur * a.nchunks, a.nchunks, s_parts);
-        if (t == 0) S.final_l1 = fv;
+        if (t == 0) st->final_l1 = fv;
     }
     __syncthreads();
     if (t < SW) ((unsigned *)st)[t] = ((const unsigned *)&S)[t];
