@@ -449,49 +449,14 @@ __global__ void k_csr_sort(int m, const int32_t *rowptr, int32_t *colidx)
 
 // Def. GM items 4 and 6.  Row i: sum of x over its columns (ascending) in FP64,
 // plus sigma_n times a Box-Muller deviate of Philox block (0, i, 0, 'N'),
-// rounded to FP32 once.  A CTA takes 32 rows: its eight warps read and gather
-// 32 entries of each row (a row's column ids are consecutive) into shared memory,
-// 256 entries of every row at a time, with a mask of the nonzero ones; lane l of
-// warp 0 then adds row l's in ascending order (skipping zeros changes no sum).
-// One thread per row read its own ids one by one.
-#define RL0_SK_WARPS 8
-__global__ void __launch_bounds__(32 * RL0_SK_WARPS) k_sketch(int m, const int32_t *rowptr, const int32_t *colidx,
-                                                              const float *x, double sigma_n, uint32_t k0, uint32_t k1,
-                                                              float *y)
+// rounded to FP32 once.
+__global__ void k_sketch(int m, const int32_t *rowptr, const int32_t *colidx, const float *x, double sigma_n,
+                         uint32_t k0, uint32_t k1, float *y)
 {
-    __shared__ float sh[RL0_SK_WARPS][32][33];
-    __shared__ unsigned nzm[RL0_SK_WARPS][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int i = blockIdx.x * 32 + lane;
-    // places in a row are counted from its start (unsigned: a place past a row's end, up to the
-    // longest row's, added to the row's start could pass 2^31)
-    const int32_t b = (i < m) ? rowptr[i] : 0;
-    const unsigned len = (i < m) ? (unsigned)(rowptr[i + 1] - b) : 0u;
-    const unsigned longest = __reduce_max_sync(0xffffffffu, len);
-    double acc = 0.0;
-    for (unsigned c0 = 0; c0 < longest; c0 += 32 * RL0_SK_WARPS) {
-        const unsigned c = c0 + 32 * wid;
-        unsigned mine = 0u;                         // lane q: the nonzero entries of row q
-        if (c < longest) {
-#pragma unroll 16
-            for (int q = 0; q < 32; ++q) {
-                const int32_t rb = __shfl_sync(0xffffffffu, b, q);
-                const unsigned rl = __shfl_sync(0xffffffffu, len, q), p = c + lane;
-                const float v = (p < rl) ? __ldg(x + __ldg(colidx + rb + p)) : 0.0f;
-                const unsigned nz = __ballot_sync(0xffffffffu, v != 0.0f);
-                if (nz) sh[wid][q][lane] = v;
-                if (lane == q) mine = nz;
-            }
-        }
-        nzm[wid][lane] = mine;
-        __syncthreads();
-        if (wid == 0)
-            for (int w = 0; w < RL0_SK_WARPS; ++w)
-                for (unsigned nz = nzm[w][lane]; nz; nz &= nz - 1u) acc += (double)sh[w][lane][__ffs(nz) - 1];
-        __syncthreads();
-    }
-    if (wid != 0) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
+    double acc = 0.0;
+    for (int32_t p = rowptr[i]; p < rowptr[i + 1]; ++p) acc += (double)x[colidx[p]];
     if (sigma_n > 0.0) {
         PhiloxOut o = philox4x32_10(0u, (uint32_t)i, 0u, TAG_NOISE, k0, k1);
         const double u1 = ((double)o.v[0] + 1.0) / 4294967296.0;
@@ -715,7 +680,7 @@ extern "C" int rl0_sketch(const rl0_expander *A, const float *x_dev, double sigm
     if (!A || !x_dev || !y_dev || !(sigma_n >= 0.0)) return RL0_ERR_INVALID_ARG;
     int rc = rl0_set_device_of(A);
     if (rc) return rc;
-    k_sketch<<<rl0_div_up(A->m, 32), 32 * RL0_SK_WARPS, 0, (cudaStream_t)cuda_stream>>>(
+    k_sketch<<<rl0_div_up(A->m, 256), 256, 0, (cudaStream_t)cuda_stream>>>(
         (int)A->m, A->rowptr, A->colidx, x_dev, sigma_n, (uint32_t)noise_seed, (uint32_t)(noise_seed >> 32), y_dev);
     CK(cudaGetLastError());
     return RL0_OK;
